@@ -248,7 +248,7 @@ struct HugeArgs {
 // Exclusive scan of the bin totals (one CTA); list of bins too large for the
 // shared-memory bin build (huge ones split into segments); closing CSR
 // offset offsets[V] = n; with wide_count, the number of bins of more than
-// wide_lo and at most emax edges (the bin build's single-buffered launch).
+// wide_lo and at most emax edges (the bin build's second launch).
 __global__ void __launch_bounds__(1024) k_scan_bins(const uint32_t* __restrict__ T, uint32_t nbins,
                                                     uint32_t* __restrict__ BS, uint32_t emax,
                                                     uint32_t* __restrict__ ovf_list,
@@ -520,10 +520,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map 
   }
 }
 
-// Phase 3: build every bin in shared memory.  Persistent CTAs (one or two
-// per SM) take bins round-robin; with two staging buffers the next bin's
-// keys and ids are fetched by TMA while the current one is sorted.  Bins
-// above emax are skipped here.
+// Phase 3: build every bin in shared memory.  Persistent CTAs take bins
+// round-robin; bins above emax are skipped here.
 template <typename K>
 struct BinArgs {
   const K* in_k;
@@ -535,405 +533,486 @@ struct BinArgs {
   const uint32_t* BS;
   uint64_t V;
   uint32_t nbins, s, emax;
+  uint32_t list;      // bins one CTA may take (room in its bin list)
   uint32_t emin;      // bins of at most emin edges are another launch's; 0: no lower bound (empty
                       // bins are built too: their buckets' offsets must be written)
   uint32_t pos_base;  // added to every offset written (position of element 0 in the CSR arrays)
-  int nbuf;  // staging buffers: 2 = next bin prefetched during this one
-  uint32_t* status;
+  bool has_pos;           // room for bin positions: the launch can rank by position
   const uint32_t* order;  // order mode word (null: partitions were stable); see k_partition
-  const uint32_t* gate;  // null, or a count written by k_scan_bins: the launch returns when it is 0
+  const uint32_t* gate;   // null, or a count written by k_scan_bins: no bin for the launch when it is 0
 };
 
-// Whether the bin build recomputes an edge's bucket rather than keeping it
-// in shared memory between its two uses (cheap maps only).
-template <typename Map>
-struct recompute_bucket {
-  static constexpr bool value = false;
-};
-template <>
-struct recompute_bucket<MurmurMap> {
-  static constexpr bool value = true;
-};
+// Edges per thread of the bin build: a CTA of NT threads builds bins of up to
+// NT * bin_ipt<K>() edges (9216 uint32 or 7168 uint64 edges with 512 threads).
+template <typename K>
+__host__ __device__ constexpr int bin_ipt() {
+  return sizeof(K) == 8 ? 14 : 18;
+}
+constexpr uint32_t kBinInfo = 255;   // longest bucket whose length and arrival ranks fit one slot's 16 bits
+constexpr uint32_t kBinBitmaps = 4;  // warps (and bitmaps) ranking longer buckets of stable partitions
+constexpr int kBinUnroll = 6;        // comparisons of a bucket made without a loop
 
-
-// Sorts the slots opos[beg, end) of one bucket (end - beg <= 32 * KR) by
-// position, with one warp: every lane holds up to KR positions, counts the
-// bucket's positions below each of them (all lanes read the same slot, a
-// broadcast) and, once every lane has read them all, stores each at its rank.
-// Positions are distinct, so the ranks are a permutation of the slots.
-template <int KR>
-__device__ __forceinline__ void warp_rank_positions(uint16_t* opos, uint32_t beg, uint32_t end, uint32_t lane) {
-  uint32_t p[KR], r[KR];
-#pragma unroll
-  for (int k = 0; k < KR; ++k) {
-    const uint32_t i = beg + lane + 32u * k;
-    p[k] = i < end ? (uint32_t)opos[i] : 0xffffffffu;
-    r[k] = 0;
-  }
-  for (uint32_t i = beg; i < end; ++i) {
-    const uint32_t x = opos[i];
-#pragma unroll
-    for (int k = 0; k < KR; ++k) r[k] += x < p[k];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < KR; ++k)
-    if (beg + lane + 32u * k < end) opos[beg + r[k]] = (uint16_t)p[k];
-  __syncwarp();
+// Shared memory of k_binbuild: the bin's keys and ids in bucket order (and up
+// to 3 entries before them), packed u16 bucket counters, the CTA's list of
+// `list` bins, and two bytes per edge for the bucket list or the slot words;
+// with pos also the bin positions, and the list and bitmaps of long buckets.
+__host__ __device__ inline uint32_t bin_cnt_words(uint32_t s) {  // one more counter than buckets, whole 16-byte pieces
+  return (uint32_t)((((size_t)1 << s) + 2) / 2 + 3) & ~3u;
+}
+__host__ __device__ inline uint32_t bin_map_words(uint32_t emax) { return (emax + 31) / 32; }
+static size_t bin_smem_bytes(int kb, uint32_t emax, uint32_t s, uint32_t list, bool pos) {
+  size_t b = (size_t)(emax + 4) * (kb + 4) + (size_t)emax * 2 + (size_t)bin_cnt_words(s) * 4 + 32 * 4 + 16 +
+             2 * (size_t)list * 4;
+  if (pos) b += (size_t)emax * 2 + kBinBitmaps * (size_t)bin_map_words(emax) * 6 + (emax / (kBinInfo + 1) + 1) * 2;
+  return align_up(b, 16);
 }
 
-// The same ranking by id instead of bin position, for bins whose tiles were
-// partitioned in any order (the ids are then input positions, distinct):
-// every lane holds up to KR (slot, id) pairs, counts the bucket's ids below
-// each of them (all lanes read the same slot and id, broadcasts) and stores
-// each slot at its rank.
-template <int KR>
-__device__ __forceinline__ void warp_rank_ids(uint16_t* opos, const uint32_t* ii, uint32_t beg, uint32_t end,
-                                              uint32_t lane) {
-  uint32_t p[KR], id[KR], r[KR];
-#pragma unroll
-  for (int k = 0; k < KR; ++k) {
-    const uint32_t i = beg + lane + 32u * k;
-    p[k] = i < end ? (uint32_t)opos[i] : 0u;
-    id[k] = i < end ? ii[p[k]] : 0xffffffffu;
-    r[k] = 0;
-  }
-  for (uint32_t i = beg; i < end; ++i) {
-    const uint32_t x = ii[opos[i]];
-#pragma unroll
-    for (int k = 0; k < KR; ++k) r[k] += x < id[k];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int k = 0; k < KR; ++k)
-    if (beg + lane + 32u * k < end) opos[beg + r[k]] = (uint16_t)p[k];
-  __syncwarp();
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {  // whole 16-byte pieces inside [p, p + bytes)
+  const uintptr_t a = ((uintptr_t)p + 15) & ~(uintptr_t)15, e = ((uintptr_t)p + bytes) & ~(uintptr_t)15;
+  if (e > a)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((uint32_t)(e - a)) : "memory");
 }
 
-// Compile-time switches (the defaults are the measured choices): the
-// single-buffered second bin-build launch for bins above the double-buffered
-// size, and the register ranking by id of buckets of 33 .. kBinRankBucket
-// edges when the partitions ranked tiles in any order.
-#ifndef HG_BIN_WIDE
-#define HG_BIN_WIDE 1
-#endif
-#ifndef HG_ANY_WARP_RANK
-#define HG_ANY_WARP_RANK 1
-#endif
-
-// Shared memory of k_binbuild: staging buffers of keys and ids, the local
-// bucket array (LB), slot order (u16), packed u16 bucket counters, the list
-// of long buckets, kBinBitmapWarps position bitmaps and small control state.
-size_t bin_smem_bytes(int kb, uint32_t emax, uint32_t s, int nbuf, bool lb) {
-  size_t b = (size_t)nbuf * (emax + 16) * (kb + 4) + (lb ? (size_t)emax * 2 : 0) + (size_t)emax * 2 +
-             (((size_t)1 << s) + 1) / 2 * 4 + ((size_t)emax / (kBinSmallBucket + 1) + 2) * 2;
-  b = align_up(b, 16) + (size_t)kBinBitmapWarps * ((emax + 31) / 32) * 4;
-  return align_up(b, 16) + 32 * 4 + 16 + 2 * kMaxBinsPerCta * 4 + 2 * 8 + 64;
+// Copies n elements from shared to global memory in 16-byte pieces: src is
+// 16-byte aligned, element i lies at src[shift + i], and dst - shift is
+// 16-byte aligned.
+template <int NT, typename T>
+__device__ __forceinline__ void copy_out(T* __restrict__ dst, const T* src, uint32_t shift, uint32_t n) {
+  constexpr uint32_t P = 16 / sizeof(T);
+  const uint32_t pieces = (shift + n + P - 1) / P;
+  for (uint32_t v = threadIdx.x; v < pieces; v += NT) {
+    const uint32_t i = v * P;
+    if (i >= shift && i + P <= shift + n) {
+      *reinterpret_cast<uint4*>(dst + (i - shift)) = *reinterpret_cast<const uint4*>(src + i);
+    } else {
+      for (uint32_t k = i; k < i + P; ++k)
+        if (k >= shift && k < shift + n) dst[k - shift] = src[k];
+    }
+  }
 }
 
 // Per bin (E <= emax edges, nb local buckets):
-//   1. local bucket of every edge; bucket counts by shared-memory atomics
-//      (counts do not depend on order); two 16-bit counters per word
-//   2. exclusive scan of the counts -> bucket starts, packed the same way
-//   3. every edge claims a slot of its bucket with an atomic increment; the
-//      slot order inside a bucket is arbitrary at this point
-//   4. buckets above kBinSmallBucket edges sort their slots by position in
-//      the bin: up to kBinRankBucket edges one warp ranks a bucket's
-//      positions in registers, longer buckets use per-warp position bitmaps;
-//      the position is input order when both partition passes were stable
-//   5. the edges are written out in slot order, and the bin's offsets
-//      (both coalesced)
-// LB: the local buckets of step 1 are kept for step 3 (else recomputed).
-// ANY: the partitions ranked tiles in any order (see k_partition), so the
-// bin positions no longer follow the input order; every bucket of two or
-// more edges is then ranked by id (an input position, distinct) instead:
-// in registers by one warp for 33 .. kBinRankBucket edges (step 4), edge by
-// edge otherwise (step 5).
+//   1. local bucket of every edge; a shared-memory atomic on the bucket's
+//      counter (two 16-bit counters per word) counts it and gives the edge
+//      its arrival rank in the bucket; (bucket, rank) stays in a register
+//   2. exclusive scan of the counts -> bucket starts, packed the same way,
+//      and a list of the buckets of two or more edges
+//   3. every edge goes to slot (bucket start + arrival rank) in shared
+//      memory; the bin's offsets are written, coalesced
+//   4. the buckets are put in canonical order, ascending id (order mode 0:
+//      the ids are input positions, distinct) or bin position (stable
+//      partitions: bin positions follow the input), and written out
+// Step 4, where the order is by id and few buckets are long (the usual case
+// at load 1): one thread sorts a bucket of up to 4 edges in registers, one
+// warp a bucket of up to 32 edges, in place in shared memory; then keys and
+// ids leave as straight 16-byte copies.  Else ("dense"): every slot gets a
+// 16-bit word of its bucket's length and its own arrival rank in step 3, and
+// the edge of each slot goes straight to its place, the number of its
+// bucket's edges with a smaller id or position; neighbouring slots hold
+// neighbouring buckets, so these reads and the stores are coalesced.
+// Buckets above kBinInfo edges find their range through the map again; with
+// stable partitions they get their places from a bitmap of their positions
+// (a prefix count) instead of comparisons.
 // A bin takes this kernel when E <= emax and, for emin > 0, E > emin: one
-// launch (emin = 0) covers every bin that fits its double-buffered staging,
-// empty ones included, a second, single-buffered launch (twice the staging
-// room) the larger ones up to its own emax.
-template <typename K, typename Map, int NWB, int MINB, bool LB, bool ANY>
-__global__ void __launch_bounds__(NWB * 32, MINB) k_binbuild(BinArgs<K> a, Map map) {
-  if (a.order != nullptr && ((*(volatile const uint32_t*)a.order == 0u) != ANY)) return;
-  if (a.gate != nullptr && *(volatile const uint32_t*)a.gate == 0u) return;  // no bin for this launch
-  constexpr uint32_t NBM = kBinBitmapWarps;
-  const uint32_t EB = a.emax + 16;
-  const int nbuf = a.nbuf;
+// launch (emin = 0) covers every bin of the expected size, empty ones
+// included, a second one with the largest CTAs the larger ones up to its own
+// emax, and every bin when the order mode asks for positions the first
+// launch has no room for.
+//
+// Bound by instruction issue and shared-memory accesses, not HBM: keys are
+// loaded twice and ids once, in whole warps, straight to registers, from L2
+// (the next bin is prefetched there).  Several CTAs per SM (1024 threads in
+// all) overlap one bin's loads and barriers with another's work.  Measured
+// with uint32 keys at load 1, against one 1024-thread CTA per SM that staged
+// bins by TMA, claimed slots in a second round of atomics and gathered every
+// edge through a slot list: 1.61 against 2.38 ms at 2^28 keys (bins of 8192),
+// 0.76 against 1.51 ms at 2^27 (bins of 4096).  ncu at 2^26: 126 instructions
+// per 32 edges (issue active 53%) and shared-memory wavefronts 69% of peak.
+template <typename K, typename Map, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_binbuild(BinArgs<K> a, Map map) {
+  constexpr int IPT = bin_ipt<K>();
+  constexpr int G = sizeof(K) == 8 ? 7 : 6;  // edges per thread taken together
+  static_assert(IPT % G == 0, "whole groups");
+  const bool pos = a.order == nullptr || *(volatile const uint32_t*)a.order != 0u;
+  if (pos && !a.has_pos) return;
+  uint32_t emin = a.emin;
+  if (emin != 0) {  // second launch
+    if (pos && a.order != nullptr) emin = 0;  // the first launch took no bin
+    else if (*(volatile const uint32_t*)a.gate == 0u) return;
+  }
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t* sp = smem;
-  // staging buffer b of keys at kin0 + b * EB, of ids at iin0 + b * EB
-  K* const kin0 = (K*)sp; sp += (size_t)nbuf * EB * sizeof(K);
-  uint32_t* const iin0 = (uint32_t*)sp; sp += (size_t)nbuf * EB * 4;
-  uint16_t* lb = (uint16_t*)sp; sp += LB ? (size_t)a.emax * 2 : 0;
-  uint16_t* opos = (uint16_t*)sp; sp += (size_t)a.emax * 2;
-  uint32_t* cnt = (uint32_t*)sp; sp += (((size_t)1 << a.s) + 1) / 2 * 4;
-  uint16_t* heavy = (uint16_t*)sp; sp += (size_t)(a.emax / (kBinSmallBucket + 1) + 2) * 2;
-  sp = (uint8_t*)(((uintptr_t)sp + 15) & ~(uintptr_t)15);
-  const uint32_t bm_words = (a.emax + 31) / 32;
-  uint32_t* bitmaps = (uint32_t*)sp;  // NBM bitmaps of bm_words words
-  sp += (size_t)NBM * bm_words * 4;
-  sp = (uint8_t*)(((uintptr_t)sp + 15) & ~(uintptr_t)15);
-  uint32_t* wsum = (uint32_t*)sp; sp += 32 * 4;
-  uint32_t* nheavy = (uint32_t*)sp; sp += 16;
-  uint32_t* bl_start = (uint32_t*)sp; sp += kMaxBinsPerCta * 4;  // this CTA's bins: start, size
-  uint32_t* bl_size = (uint32_t*)sp; sp += kMaxBinsPerCta * 4;
-  uint64_t* bar = (uint64_t*)sp;
+  K* const ks0 = (K*)sp; sp += (size_t)(a.emax + 4) * sizeof(K);
+  uint32_t* const is0 = (uint32_t*)sp; sp += (size_t)(a.emax + 4) * 4;
+  uint32_t* const cnt = (uint32_t*)sp; sp += (size_t)bin_cnt_words(a.s) * 4;
+  const uint16_t* const cnt16 = (const uint16_t*)cnt;
+  uint32_t* const wsum = (uint32_t*)sp; sp += 32 * 4;
+  uint32_t* const nlong = (uint32_t*)sp; sp += 16;  // [0] buckets of 5 .. 32 edges + 2^16 * longer; [1] buckets above kBinInfo
+  uint32_t* const bl_start = (uint32_t*)sp; sp += (size_t)a.list * 4;  // this CTA's bins: start, size
+  uint32_t* const bl_size = (uint32_t*)sp; sp += (size_t)a.list * 4;
+  uint32_t* const multi = (uint32_t*)sp;  // buckets of 2 or more edges: start | length << 16 (at most emax / 2)
+  uint16_t* const info = (uint16_t*)sp; sp += (size_t)a.emax * 2;  // dense: length | arrival rank << 8; 0: longer
+  // used only with pos (sizes: whole words)
+  uint16_t* const ps = (uint16_t*)sp; sp += (size_t)a.emax * 2;
+  const uint32_t map_words = bin_map_words(a.emax);
+  uint32_t* const hbits = (uint32_t*)sp; sp += kBinBitmaps * (size_t)map_words * 4;
+  uint16_t* const hpre = (uint16_t*)sp; sp += kBinBitmaps * (size_t)map_words * 2;
+  uint16_t* const heavy = (uint16_t*)sp;
 
   map.init();
-  const uint32_t koff = align_first<sizeof(K)>(a.in_k), ioff = align_first<4>(a.in_i);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   // Bins blockIdx.x, +gridDim.x, ...: starts and sizes gathered once, so the
   // loop below needs no global loads to find its next bin.
   const uint32_t nmine = blockIdx.x < a.nbins ? (a.nbins - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
-  for (uint32_t j = threadIdx.x; j < nmine; j += blockDim.x) {
+  for (uint32_t j = tid; j < nmine; j += NT) {
     const uint32_t bb = blockIdx.x + j * gridDim.x;
     bl_start[j] = a.BS[bb];
     bl_size[j] = a.T[bb];
   }
+  const uint32_t cnt_words = bin_cnt_words(a.s);
+  for (uint32_t w = tid; w < cnt_words; w += NT) cnt[w] = 0;
+  if (tid < 2) nlong[tid] = 0;
   __syncthreads();
-  auto skip = [&](uint32_t j) {
-    while (j < nmine && (bl_size[j] > a.emax || (a.emin != 0 && bl_size[j] <= a.emin))) ++j;
+  auto skip = [&](uint32_t j) {  // the CTA's first bin from its j-th on that this launch takes
+    while (j < nmine && (bl_size[j] > a.emax || (emin != 0 && bl_size[j] <= emin))) ++j;
     return j;
   };
-  auto issue = [&](uint32_t j, int buf) {
-    if (threadIdx.x == 0) {
-      const uint64_t k0 = bl_start[j], k1 = k0 + bl_size[j];
-      const TileSpan<sizeof(K)> sk_ = tile_span<sizeof(K)>(koff, k0, k1);
-      const TileSpan<4> si_ = tile_span<4>(ioff, k0, k1);
-      mbar_arrive_expect_tx(&bar[buf], sk_.bytes() + si_.bytes());
-      if (sk_.body) tma_load_1d(kin0 + (size_t)buf * EB + sk_.dst(), a.in_k + sk_.b0, sk_.bytes(), &bar[buf]);
-      if (si_.body) tma_load_1d(iin0 + (size_t)buf * EB + si_.dst(), a.in_i + si_.b0, si_.bytes(), &bar[buf]);
-    }
-  };
-  if (threadIdx.x == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
   uint32_t jb = skip(0);
-  if (jb >= nmine) return;
-  issue(jb, 0);
-  const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-  for (uint32_t it = 0; jb < nmine; ++it) {
-    const uint32_t b = blockIdx.x + jb * gridDim.x;
-    const int buf = nbuf == 2 ? (int)(it & 1) : 0;
-    const uint32_t jb_next = skip(jb + 1);
-    if (nbuf == 2 && jb_next < nmine) issue(jb_next, buf ^ 1);
-    const uint64_t bucket0 = (uint64_t)b << a.s;
-    const uint32_t nb = (uint32_t)min((uint64_t)1 << a.s, a.V - bucket0);
-    const uint32_t nwords = (nb + 1) >> 1;
-    for (uint32_t w = threadIdx.x; w < nwords; w += blockDim.x) cnt[w] = 0;
-    if (threadIdx.x == 0) *nheavy = 0;
-    const uint32_t parity = nbuf == 2 ? (it >> 1) & 1u : it & 1u;
-    if (!mbar_wait_block(&bar[buf], parity, a.status)) return;
+  while (jb < nmine) {
     const uint32_t E = bl_size[jb], start = bl_start[jb];
-    const TileSpan<sizeof(K)> sk_ = tile_span<sizeof(K)>(koff, start, (uint64_t)start + E);
-    const TileSpan<4> si_ = tile_span<4>(ioff, start, (uint64_t)start + E);
-    K* const kb_ = kin0 + (size_t)buf * EB;
-    uint32_t* const ib_ = iin0 + (size_t)buf * EB;
-    load_edges<sizeof(K)>(kb_, a.in_k, sk_);
-    load_edges<4>(ib_, a.in_i, si_);
-    if (sk_.edges() || si_.edges())
-      __syncthreads();  // edge elements came in by plain loads (block-uniform condition)
-    const K* kk = kb_ + sk_.lead();
-    const uint32_t* ii = ib_ + si_.lead();
-    // 1. local buckets and counts
-    for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-      const uint32_t l = map(kk[e], ii[e]) - (uint32_t)bucket0;
-      if (LB) lb[e] = (uint16_t)l;
-      atomicAdd(&cnt[l >> 1], 1u << ((l & 1u) << 4));
+    const uint64_t bucket0 = (uint64_t)(blockIdx.x + jb * gridDim.x) << a.s;
+    const uint32_t nb = (uint32_t)min((uint64_t)1 << a.s, a.V - bucket0);
+    jb = skip(jb + 1);
+    if (tid == 0 && jb < nmine) {
+      prefetch_l2(a.in_k + bl_start[jb], bl_size[jb] * (uint32_t)sizeof(K));
+      prefetch_l2(a.in_i + bl_start[jb], bl_size[jb] * 4u);
     }
+    // edge tid + c * NT of the bin is this thread's when left > c * NT
+    const int left = (int)E - (int)tid;
+    const K* const gk = a.in_k + start + tid;
+    const uint32_t* const gi = a.in_i + start + tid;
+    K key[G];
+    uint32_t id[G];
+    auto load_keys = [&](int g) {  // of the edges g .. g + G - 1
+#pragma unroll
+      for (int u = 0; u < G; ++u) key[u] = left > (g + u) * NT ? __ldg(gk + (g + u) * NT) : K(0);
+    };
+    auto load_ids = [&](int g) {
+#pragma unroll
+      for (int u = 0; u < G; ++u) id[u] = left > (g + u) * NT ? __ldg(gi + (g + u) * NT) : 0u;
+    };
+    // a group of edges through f(c, u): whole groups without a test per edge
+    auto group = [&](int g, auto&& f) {
+      if ((uint32_t)(g + G) * NT <= E) {  // block-uniform
+#pragma unroll
+        for (int u = 0; u < G; ++u) f(g + u, u);
+      } else {
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+          if (left > (g + u) * NT) f(g + u, u);
+      }
+    };
+    // 1. local buckets, counts, arrival ranks
+    uint32_t br[IPT];  // bucket | rank << 16
+#pragma unroll
+    for (int g = 0; g < IPT; g += G) {
+      if ((uint32_t)g * NT >= E) break;  // block-uniform
+      load_keys(g);
+      if (Map::kNeedsPos) load_ids(g);
+      group(g, [&](int c, int u) {
+        const uint32_t l = map(key[u], Map::kNeedsPos ? id[u] : 0u) - (uint32_t)bucket0;
+        const uint32_t odd = l & 1u;
+        const uint32_t old = atomicAdd(&cnt[l >> 1], 1u + odd * 0xffffu);
+        br[c] = __byte_perm(l, old, 0x5410u + odd * 0x2200u);  // the bucket's half of old above l
+      });
+    }
+    load_keys(0);  // for step 3: these arrive during the scan
+    load_ids(0);
     __syncthreads();
-    // 2. exclusive scan of the counts; buckets above kBinSmallBucket edges
-    //    are listed for the bitmap sort
+    // 2. exclusive scan of the counts (a thread's counts sum to at most E < 2^15)
+    uint32_t nmulti;
     {
-      const uint32_t per = (nwords + blockDim.x - 1) / blockDim.x;
-      const uint32_t w0 = min(threadIdx.x * per, nwords), w1 = min(w0 + per, nwords);
-      uint32_t sum = 0;
-      for (uint32_t w = w0; w < w1; ++w) {
-        const uint32_t x = cnt[w];
-        sum += (x & 0xffffu) + (x >> 16);
+      const uint32_t words = (nb + 2) >> 1;  // the counter after the last bucket's receives E
+      const uint32_t per = ((words + NT - 1) / NT + 3u) & ~3u;  // words per thread, whole 16-byte pieces
+      const uint32_t w0 = min(tid * per, cnt_words), w1 = min(w0 + per, cnt_words);
+      // of the two counters of a word: flags of those of at least m edges
+      auto at_least = [](uint32_t x, uint32_t m) { return (x + (0x8000u - m) * 0x10001u) & 0x80008000u; };
+      uint32_t sum = 0, two = 0, five = 0, big = 0;
+      for (uint32_t w = w0; w < w1; w += 4) {
+        const uint4 x = *reinterpret_cast<const uint4*>(cnt + w);
+        sum += x.x + x.y + x.z + x.w;  // both halves at once
+        two += __popc(at_least(x.x, 2) | (at_least(x.y, 2) >> 1) | (at_least(x.z, 2) >> 2) | (at_least(x.w, 2) >> 3));
+        five += __popc(at_least(x.x, 5) | (at_least(x.y, 5) >> 1) | (at_least(x.z, 5) >> 2) | (at_least(x.w, 5) >> 3));
+        big |= at_least(x.x, 33) | at_least(x.y, 33) | at_least(x.z, 33) | at_least(x.w, 33);
       }
-      uint32_t base = block_excl_scan_nt<uint32_t>(sum, wsum);
-      for (uint32_t w = w0; w < w1; ++w) {
-        const uint32_t x = cnt[w], lo = x & 0xffffu, hi = x >> 16;
-        if ((HG_ANY_WARP_RANK || !ANY) && lo > kBinSmallBucket) heavy[atomicAdd(nheavy, 1u)] = (uint16_t)(2 * w);
-        if ((HG_ANY_WARP_RANK || !ANY) && hi > kBinSmallBucket) heavy[atomicAdd(nheavy, 1u)] = (uint16_t)(2 * w + 1);
-        cnt[w] = base | ((base + lo) << 16);
-        base += lo + hi;
+      if (five) atomicAdd(nlong, big ? 0x10000u : five);
+      const uint32_t v = ((sum & 0xffffu) + (sum >> 16)) | (two << 16);
+      uint32_t base = block_excl_scan_nt<uint32_t>(v, wsum), at = base >> 16;
+      nmulti = wsum[NT / 32 - 1] >> 16;
+      base &= 0xffffu;
+      for (uint32_t w = w0; w < w1; w += 4) {
+        uint4 x = *reinterpret_cast<const uint4*>(cnt + w);
+        auto word = [&](uint32_t c) {
+          const uint32_t lo = c & 0xffffu, hi = c >> 16, mid = base + lo;
+          const uint32_t out = __byte_perm(base, mid, 0x5410u);
+          if (lo > 1) multi[at++] = base | (lo << 16);
+          if (hi > 1) multi[at++] = mid | (c & 0xffff0000u);
+          base = mid + hi;
+          return out;
+        };
+        x.x = word(x.x);
+        x.y = word(x.y);
+        x.z = word(x.z);
+        x.w = word(x.w);
+        *reinterpret_cast<uint4*>(cnt + w) = x;
       }
     }
     __syncthreads();
-    // 3. slots
-    for (uint32_t e = threadIdx.x; e < E; e += blockDim.x) {
-      const uint32_t l = LB ? (uint32_t)lb[e] : map(kk[e], ii[e]) - (uint32_t)bucket0;
-      const uint32_t sh = (l & 1u) << 4;
-      const uint32_t old = atomicAdd(&cnt[l >> 1], 1u << sh);
-      opos[(old >> sh) & 0xffffu] = (uint16_t)e;
-    }
-    __syncthreads();
-    // 4. long buckets (every counter now holds its bucket's end): slots
-    //    sorted by position, in registers by one warp per bucket (every warp
-    //    takes buckets) up to kBinRankBucket edges, else with per-warp
-    //    position bitmaps on the first NBM warps
-    const uint32_t nh = *nheavy;
-    if (nh > 0) {
-      const uint32_t nw = blockDim.x >> 5;
-      for (uint32_t h = warp; h < nh; h += nw) {
-        const uint32_t v = heavy[h];
-        const uint32_t end = (cnt[v >> 1] >> ((v & 1u) << 4)) & 0xffffu;
-        const uint32_t beg = v ? (cnt[(v - 1) >> 1] >> (((v - 1) & 1u) << 4)) & 0xffffu : 0u;
-        if (ANY) {  // by id; longer buckets are ranked edge by edge in step 5
-          if (end - beg <= 64) warp_rank_ids<2>(opos, ii, beg, end, lane);
-          else if (end - beg <= 128) warp_rank_ids<4>(opos, ii, beg, end, lane);
-          else if (end - beg <= kBinRankBucket) warp_rank_ids<kBinRankBucket / 32>(opos, ii, beg, end, lane);
-        } else {
-          if (end - beg <= 64) warp_rank_positions<2>(opos, beg, end, lane);
-          else if (end - beg <= 128) warp_rank_positions<4>(opos, beg, end, lane);
-          else if (end - beg <= kBinRankBucket) warp_rank_positions<kBinRankBucket / 32>(opos, beg, end, lane);
-        }
+    // block-uniform: too many or too long buckets for sorting them one by one
+    const bool dense = pos || *nlong > E / 64;
+    K* const ok = a.csr_k + start;
+    uint32_t* const oi = a.csr_i + start;
+    const uint32_t shk = dense ? 0u : (uint32_t)((uintptr_t)ok & 15u) / (uint32_t)sizeof(K);
+    const uint32_t shi = dense ? 0u : (uint32_t)((uintptr_t)oi & 15u) / 4u;
+    K* const ks = ks0 + shk;
+    uint32_t* const is = is0 + shi;
+    // 3. edges to their slots; offsets
+#pragma unroll
+    for (int g = 0; g < IPT; g += G) {
+      if ((uint32_t)g * NT >= E) break;
+      if (g > 0) {
+        load_keys(g);
+        load_ids(g);
       }
-    }
-    if (!ANY && nh > 0 && warp < NBM) {
-      // each of the first NBM warps owns one bitmap of E bits
-      const uint32_t nbits_words = (E + 31) >> 5;
-      uint32_t* bm = bitmaps + warp * bm_words;
-      for (uint32_t h = warp; h < nh; h += NBM) {
-        const uint32_t v = heavy[h];
-        const uint32_t end = (cnt[v >> 1] >> ((v & 1u) << 4)) & 0xffffu;
-        const uint32_t beg = v ? (cnt[(v - 1) >> 1] >> (((v - 1) & 1u) << 4)) & 0xffffu : 0u;
-        if (end - beg <= kBinRankBucket) continue;  // ranked above
-        for (uint32_t k = lane; k < nbits_words; k += 32) bm[k] = 0;
-        __syncwarp();
-        for (uint32_t i = beg + lane; i < end; i += 32) {
-          const uint32_t p = opos[i];
-          atomicOr(&bm[p >> 5], 1u << (p & 31u));
-        }
-        __syncwarp();
-        uint32_t run = beg;
-        for (uint32_t k0 = 0; k0 < nbits_words; k0 += 32) {
-          uint32_t word = k0 + lane < nbits_words ? bm[k0 + lane] : 0u;
-          const uint32_t c = __popc(word);
-          const uint32_t incl = warp_incl_scan(c);
-          uint32_t pos = run + incl - c;
-          while (word) {
-            const uint32_t bit = __ffs(word) - 1;
-            opos[pos++] = (uint16_t)(((k0 + lane) << 5) + bit);
-            word &= word - 1;
+      if (!dense) {
+        group(g, [&](int c, int u) {
+          const uint32_t slot = cnt16[br[c] & 0xffffu] + (br[c] >> 16);
+          ks[slot] = key[u];
+          is[slot] = map.out_id(id[u]);
+        });
+      } else {
+        group(g, [&](int c, int u) {
+          const uint32_t l = br[c] & 0xffffu, r = br[c] >> 16;
+          const uint32_t beg = cnt16[l], n = cnt16[l + 1] - beg;
+          const uint32_t slot = beg + r;
+          ks[slot] = key[u];
+          is[slot] = id[u];
+          info[slot] = (uint16_t)(n <= kBinInfo ? n | (r << 8) : 0u);
+          if (pos) {
+            ps[slot] = (uint16_t)(tid + c * NT);
+            if (r == kBinInfo) heavy[atomicAdd(nlong + 1, 1u)] = (uint16_t)l;  // one edge of every longer bucket
           }
-          run += __shfl_sync(kFull, incl, 31);
-        }
-        __syncwarp();
+        });
       }
     }
-    if (nh > 0) __syncthreads();  // block-uniform: every thread read the same count
-    // 5. edges in canonical order: the edge in slot j of a bucket of at most
-    //    kBinSmallBucket edges goes to the bucket's start plus the number of
-    //    its edges with a smaller position (positions are distinct, so the
-    //    ranks are a permutation of the bucket's slots; the stores of a warp
-    //    stay within a few sectors); a long bucket is already in order.  With
-    //    ANY every bucket is ranked by id the same way.
-    //    Then the bin's offsets (bucket v starts where bucket v - 1 ends).
-    // Whether slot j's bucket [beg, end) still needs ranking here (longer
-    // ones were put in order in step 4), and its rank.
-    auto loose = [&](uint32_t beg, uint32_t end) {
-      const uint32_t n = end - beg;
-      if (n < 2) return false;
-      if (ANY) return !HG_ANY_WARP_RANK || n <= kBinSmallBucket || n > kBinRankBucket;
-      return n <= kBinSmallBucket;
-    };
-    auto rank_of = [&](uint32_t beg, uint32_t end, uint32_t p, uint32_t id) {
-      uint32_t dst = beg;
-      if (ANY)
-        for (uint32_t i = beg; i < end; ++i) dst += ii[opos[i]] < id;
-      else
-        for (uint32_t i = beg; i < end; ++i) dst += opos[i] < p;
-      return dst;
-    };
-    for (uint32_t j = threadIdx.x; j < E; j += blockDim.x) {
-      const uint32_t p = opos[j];
-      const K key = kk[p];
-      const uint32_t id = ii[p];
-      const uint32_t l = LB ? (uint32_t)lb[p] : map(key, id) - (uint32_t)bucket0;
-      const uint32_t end = (cnt[l >> 1] >> ((l & 1u) << 4)) & 0xffffu;
-      const uint32_t beg = l ? (cnt[(l - 1) >> 1] >> (((l - 1) & 1u) << 4)) & 0xffffu : 0u;
-      const uint32_t dst = loose(beg, end) ? rank_of(beg, end, p, id) : j;
-      a.csr_k[start + dst] = key;
-      a.csr_i[start + dst] = map.out_id(id);
-    }
-    for (uint32_t v = threadIdx.x; v < nb; v += blockDim.x) {
-      const uint32_t first = v ? (cnt[(v - 1) >> 1] >> (((v - 1) & 1u) << 4)) & 0xffffu : 0u;
-      a.offsets[bucket0 + v] = a.pos_base + start + first;
+    {
+      uint32_t* const off = a.offsets + bucket0;
+      const uint32_t o = a.pos_base + start;
+      if (((uintptr_t)off & 7) == 0) {  // two buckets per store
+        for (uint32_t w = tid; w < nb >> 1; w += NT) {
+          const uint32_t x = cnt[w];
+          *reinterpret_cast<uint2*>(off + 2 * w) = make_uint2(o + (x & 0xffffu), o + (x >> 16));
+        }
+        if ((nb & 1u) && tid == 0) off[nb - 1] = o + cnt16[nb - 1];
+      } else {
+        for (uint32_t v = tid; v < nb; v += NT) off[v] = o + cnt16[v];
+      }
     }
     __syncthreads();
-    if (nbuf == 1 && jb_next < nmine) issue(jb_next, 0);
-    jb = jb_next;
+    auto clear = [&]() {
+      for (uint32_t w = tid * 4; w < cnt_words; w += NT * 4)
+        *reinterpret_cast<uint4*>(cnt + w) = make_uint4(0, 0, 0, 0);
+      if (tid < 2) nlong[tid] = 0;
+    };
+    if (!dense) {
+      // 4. buckets of 2 .. 4 edges by one thread each: (id, slot) pairs
+      //    through a sorting network, then the keys by slot; longer ones by
+      //    the warp, which ranks every lane's id against the others'
+      clear();
+      for (uint32_t t0 = warp * 32u; t0 < nmulti; t0 += NT) {
+        const uint32_t x = t0 + lane < nmulti ? multi[t0 + lane] : 0u;
+        const uint32_t beg = x & 0xffffu, n = x >> 16;
+        if (n >= 2 && n <= 4) {
+          uint32_t d[4], p[4];
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i) {
+            d[i] = i < n ? is[beg + i] : 0xffffffffu;  // no edge has this id
+            p[i] = i;
+          }
+          auto order = [&](int i, int j) {
+            const bool sw = d[i] > d[j];
+            const uint32_t di = d[i], pi = p[i];
+            d[i] = sw ? d[j] : di;
+            p[i] = sw ? p[j] : pi;
+            d[j] = sw ? di : d[j];
+            p[j] = sw ? pi : p[j];
+          };
+          order(0, 1);
+          if (n > 2) {
+            order(2, 3);
+            order(0, 2);
+            order(1, 3);
+            order(1, 2);
+          }
+          K k[4];
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i)
+            if (i < n) k[i] = ks[beg + p[i]];
+#pragma unroll
+          for (uint32_t i = 0; i < 4; ++i)
+            if (i < n) {
+              is[beg + i] = d[i];
+              ks[beg + i] = k[i];
+            }
+        }
+        for (uint32_t m = __ballot_sync(kFull, n > 4); m; m &= m - 1) {
+          const uint32_t y = __shfl_sync(kFull, x, __ffs(m) - 1);
+          const uint32_t b = y & 0xffffu, len = y >> 16;  // len <= 32
+          const bool in = lane < len;
+          const uint32_t cid = in ? is[b + lane] : 0u;
+          const K k = in ? ks[b + lane] : K(0);
+          uint32_t r = 0;
+          for (uint32_t i = 0; i < len; ++i) r += __shfl_sync(kFull, cid, i) < cid;
+          __syncwarp();
+          if (in) {
+            is[b + r] = cid;
+            ks[b + r] = k;
+          }
+        }
+      }
+      __syncthreads();
+      copy_out<NT>(ok, ks0, shk, E);
+      copy_out<NT>(oi, is0, shi, E);
+      __syncthreads();
+      continue;
+    }
+    const uint32_t nh = nlong[1];
+    // long buckets of stable partitions: the edge's place in its bucket
+    // replaces its bin position
+    if (nh > 0) {  // block-uniform
+      const uint32_t words = (E + 31) >> 5;
+      if (warp < kBinBitmaps) {
+        uint32_t* const bm = hbits + warp * map_words;
+        uint16_t* const pre = hpre + warp * map_words;
+        for (uint32_t h = warp; h < nh; h += kBinBitmaps) {
+          const uint32_t beg = cnt16[heavy[h]], end = cnt16[heavy[h] + 1];
+          for (uint32_t k = lane; k < words; k += 32) bm[k] = 0;
+          __syncwarp();
+          for (uint32_t i = beg + lane; i < end; i += 32) atomicOr(&bm[ps[i] >> 5], 1u << (ps[i] & 31u));
+          __syncwarp();
+          uint32_t run = 0;
+          for (uint32_t k0 = 0; k0 < words; k0 += 32) {
+            const uint32_t c = k0 + lane < words ? __popc(bm[k0 + lane]) : 0u;
+            const uint32_t incl = warp_incl_scan(c);
+            if (k0 + lane < words) pre[k0 + lane] = (uint16_t)(run + incl - c);
+            run += __shfl_sync(kFull, incl, 31);
+          }
+          __syncwarp();
+          for (uint32_t i = beg + lane; i < end; i += 32) {
+            const uint32_t p = ps[i];
+            ps[i] = (uint16_t)(pre[p >> 5] + __popc(bm[p >> 5] & ((1u << (p & 31u)) - 1u)));
+          }
+          __syncwarp();
+        }
+      }
+      __syncthreads();
+    }
+    // 4. dense: every slot's edge straight to its place
+    for (uint32_t j = tid; j < E; j += NT) {
+      const K k = ks[j];
+      const uint32_t cid = is[j], x = info[j];
+      uint32_t dst;
+      if (x != 0) {  // bucket of 1 .. kBinInfo edges
+        const uint32_t n = x & 0xffu;
+        dst = j - (x >> 8);
+        if (!pos) {
+          const uint32_t* const q = is + dst;
+#pragma unroll
+          for (int i = 0; i < kBinUnroll; ++i)
+            if ((uint32_t)i < n && q[i] < cid) ++dst;
+          if (n > kBinUnroll)
+            for (uint32_t i = kBinUnroll; i < n; ++i) dst += q[i] < cid;
+        } else {
+          const uint32_t p = ps[j];
+          const uint16_t* const q = ps + dst;
+#pragma unroll
+          for (int i = 0; i < kBinUnroll; ++i)
+            if ((uint32_t)i < n && q[i] < p) ++dst;
+          if (n > kBinUnroll)
+            for (uint32_t i = kBinUnroll; i < n; ++i) dst += q[i] < p;
+        }
+      } else {
+        const uint32_t l = map(k, cid) - (uint32_t)bucket0;
+        const uint32_t end = cnt16[l + 1];
+        uint32_t i = cnt16[l];
+        dst = i;
+        if (pos) {
+          dst += ps[j];
+        } else {  // four ids per load
+          for (; i & 3u; ++i) dst += is[i] < cid;
+          for (; i + 4 <= end; i += 4) {
+            const uint4 y = *reinterpret_cast<const uint4*>(is + i);
+            dst += (y.x < cid) + (y.y < cid) + (y.z < cid) + (y.w < cid);
+          }
+          for (; i < end; ++i) dst += is[i] < cid;
+        }
+      }
+      ok[dst] = k;
+      oi[dst] = map.out_id(cid);
+    }
+    __syncthreads();
+    clear();
+    __syncthreads();
   }
 }
 
-// Bin-build launch configuration: 512-thread CTAs two to an SM, single
-// buffered, when two fit with bins large enough for this build; otherwise
-// one CTA per SM (1024 threads unless 512 were asked for), double buffered
-// when that fits.
+// Bin-build launch configuration.
 struct BinCfg {
-  uint32_t tpb, per_sm, emax;
-  int nbuf;
-  bool lb;
+  uint32_t nt, grid, list, emax;
+  bool pos;
   size_t smem;
-  uint32_t emax_wide;  // largest bin of the single-buffered second launch (<= emax: none)
-  size_t smem_wide;
 };
-// Two 512-thread CTAs per SM (local buckets recomputed, no prefetch) measured
-// slower than one 1024-thread CTA that keeps them and prefetches the next bin
-// (2.42 against 2.27 ms at 2^28 keys); HG_BIN_TWO_PER_SM=1 selects them.
-#ifndef HG_BIN_TWO_PER_SM
-#define HG_BIN_TWO_PER_SM 0
-#endif
-static BinCfg bin_config(const Plan& p, bool recompute) {
+// The launch with CTAs of nt threads, as many to an SM as make 1024 threads:
+// the largest bin they can hold, at most nt * ipt edges.
+template <typename K>
+static BinCfg bin_config_for(const Plan& p, uint32_t nt, bool pos) {
   const DevInfo& di = dev_info();
   BinCfg c{};
-  if (HG_BIN_TWO_PER_SM && p.tpb != 1024 && di.smem_per_sm > 0) {
-    const bool lb = !recompute;
-    const double mean = p.nbins ? (double)p.n / (double)p.nbins : 0.0;
-    const size_t sm_cap = (size_t)di.smem_per_sm / 2 - (size_t)di.smem_reserved;
-    uint32_t e = p.emax;
-    while (e > 1024 && (bin_smem_bytes(p.kb, e, p.s, 1, lb) > sm_cap ||
-                        bin_smem_bytes(p.kb, e, p.s, 1, lb) > (size_t)di.max_smem_optin))
-      e -= 32;
-    // bins of a uniform build are Poisson: allow five standard deviations
-    if (bin_smem_bytes(p.kb, e, p.s, 1, lb) <= sm_cap && (double)e >= mean + 5.0 * std::sqrt(mean) + 16.0) {
-      c.tpb = 512;
-      c.per_sm = 2;
-      c.emax = e;
-      c.nbuf = 1;
-      c.lb = lb;
-      c.smem = bin_smem_bytes(p.kb, e, p.s, 1, lb);
-      return c;
-    }
-  }
-  c.tpb = p.tpb == 512 ? 512u : 1024u;
-  c.per_sm = 1;
-  c.emax = p.emax;
-  c.lb = true;
-  c.nbuf = 2;
-  c.smem = bin_smem_bytes(p.kb, p.emax, p.s, 2, true);
-  if (c.smem > (size_t)di.max_smem_optin) {
-    c.nbuf = 1;
-    c.smem = bin_smem_bytes(p.kb, p.emax, p.s, 1, true);
-  }
-  // the largest bin one single-buffered CTA can hold (slot indexes are 16-bit)
-  c.emax_wide = 0;
-  c.smem_wide = 0;
-  if (HG_BIN_WIDE && c.nbuf == 2 && di.max_smem_optin > 0) {
-    uint32_t e = 65504;
-    while (e > p.emax && bin_smem_bytes(p.kb, e, p.s, 1, true) > (size_t)di.max_smem_optin) e -= 32;
-    if (e > p.emax) {
-      c.emax_wide = e;
-      c.smem_wide = bin_smem_bytes(p.kb, e, p.s, 1, true);
-    }
-  }
+  c.nt = nt;
+  c.pos = pos;
+  const uint32_t per_sm = 1024 / nt;
+  c.grid = std::max<uint32_t>(std::min<uint32_t>(p.nbins, (uint32_t)di.sms * per_sm),
+                              (p.nbins + kMaxBinsPerCta - 1) / kMaxBinsPerCta);
+  c.list = (p.nbins + c.grid - 1) / c.grid;
+  const size_t cap =
+      per_sm == 1 ? (size_t)di.max_smem_optin : (size_t)di.smem_per_sm / per_sm - (size_t)di.smem_reserved;
+  uint32_t e = nt * bin_ipt<K>();
+  while (e > 32 && bin_smem_bytes(p.kb, e, p.s, c.list, pos) > cap) e -= 32;
+  c.emax = e;
+  c.smem = bin_smem_bytes(p.kb, e, p.s, c.list, pos);
   return c;
+}
+// CTAs of 256, 512 or 1024 threads, by the size bins are expected to have
+// (Poisson: mean and five standard deviations): the smaller the CTA, the
+// better its barriers are hidden by the other CTAs of the SM (uint32 keys at
+// load 1, 256 / 512 / 1024 threads: 0.202 / 0.244 / 0.312 ms at 2^25 keys,
+// 512 / 1024: 1.61 / 2.03 ms at 2^28).  Builds of at most two bins per SM
+// take the largest, which finish a bin soonest (256 bins at 2^20 keys: 18.9
+// us against 22.1 with 256 threads; 512 bins at 2^21: 30.4 against 27.5).  A
+// size asked for by the caller stands.
+template <typename K>
+static BinCfg bin_config(const Plan& p, bool by_id) {
+  if (p.tpb == 1024) return bin_config_for<K>(p, 1024, true);
+  if (p.tpb == 512) return bin_config_for<K>(p, 512, !by_id);
+  const double mean = (double)p.n * (double)(1ull << p.s) / (double)p.V;
+  const double need = mean + 5.0 * std::sqrt(mean) + 16.0;
+  if (p.nbins > 2 * (uint32_t)dev_info().sms) {
+    for (uint32_t nt : {256u, 512u}) {
+      const BinCfg c = bin_config_for<K>(p, nt, !by_id);
+      if ((double)c.emax >= need) return c;
+    }
+  }
+  return bin_config_for<K>(p, 1024, true);
 }
 
 // Streams edges [start, start + len) of a bin in tiles of kBigTile, sorts
@@ -1309,7 +1388,6 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     colscan_launch(C, p.G, p.nsb, CT, st);
   }
   const bool two = p.sshift > 0;
-  const BinCfg bc = bin_config(p, recompute_bucket<Map>::value);
   // Implicit ids are input positions, so the bin build can restore the
   // canonical order (ascending position in every bucket) from the ids
   // alone; then, unless k_scan_bins finds a bin too large for the
@@ -1317,7 +1395,11 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   // Both variants of each such kernel are launched; the one that does not
   // match the order mode returns at once.
   const bool any_order = ids == nullptr || positional_ids;
-  // bins for the single-buffered bin-build launch, counted by k_scan_bins
+  BinCfg bc = bin_config<K>(p, any_order);
+  const BinCfg bw = bin_config_for<K>(p, 1024, true);  // bins larger than bc.emax
+  bc.emax = std::min(bc.emax, bw.emax);
+  const uint32_t emax_all = bw.emax;
+  // bins for the bin build's second launch, counted by k_scan_bins
   uint32_t* const wide_count = (uint32_t*)&hdr->counters[7];
   {
     HG_TRACE("k_scan_bins", st);
@@ -1330,12 +1412,11 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     h.rowdesc = (uint32_t*)(ws + p.o_rowdesc);
     h.max_rows = p.max_rows;
     h.status = status;
-    // bins above the largest the shared-memory bin build takes (the second,
-    // single-buffered launch included) go to the oversized-bin kernels
-    k_scan_bins<<<1, 1024, 0, st>>>(T, p.nbins, BS, std::max(bc.emax, bc.emax_wide), ovf, &hdr->ovf_count,
-                                    offsets, p.V, pos_base + (uint32_t)p.n, h,
-                                    any_order ? &hdr->order_mode : nullptr, bc.emax,
-                                    bc.emax_wide > bc.emax ? wide_count : nullptr);
+    // bins above the largest the shared-memory bin build takes (the second
+    // launch included) go to the oversized-bin kernels
+    k_scan_bins<<<1, 1024, 0, st>>>(T, p.nbins, BS, emax_all, ovf, &hdr->ovf_count, offsets, p.V,
+                                    pos_base + (uint32_t)p.n, h, any_order ? &hdr->order_mode : nullptr, bc.emax,
+                                    bc.nt != bw.nt ? wide_count : nullptr);
   }
 
   PartArgs<K> pa{};
@@ -1420,40 +1501,27 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   ba.V = p.V;
   ba.nbins = p.nbins;
   ba.s = p.s;
-  ba.emax = bc.emax;
   ba.pos_base = pos_base;
-  ba.status = status;
-  ba.nbuf = bc.nbuf;
   ba.order = any_order ? &hdr->order_mode : nullptr;
   {
-    unsigned grid = (unsigned)std::min<uint64_t>(p.nbins, (uint64_t)di.sms * bc.per_sm);
-    grid = std::max<unsigned>(grid, (p.nbins + kMaxBinsPerCta - 1) / kMaxBinsPerCta);
     HG_TRACE("k_binbuild", st);
-    auto launch = [&](auto kern, auto kany, unsigned threads) {
-      set_smem_once(kern, std::max(bc.smem, bc.smem_wide));
-      set_smem_once(kany, std::max(bc.smem, bc.smem_wide));
-      if (any_order) kany<<<grid, threads, bc.smem, st>>>(ba, map);
-      kern<<<grid, threads, bc.smem, st>>>(ba, map);
-      if (bc.emax_wide > bc.emax) {  // bins above emax, single-buffered
-        BinArgs<K> bw = ba;
-        bw.emin = bc.emax;
-        bw.emax = bc.emax_wide;
-        bw.nbuf = 1;
-        bw.gate = wide_count;
-        if (any_order) kany<<<grid, threads, bc.smem_wide, st>>>(bw, map);
-        kern<<<grid, threads, bc.smem_wide, st>>>(bw, map);
-      }
+    auto launch = [&](const BinCfg& c, uint32_t emin, const uint32_t* gate) {
+      BinArgs<K> x = ba;
+      x.emax = c.emax;
+      x.list = c.list;
+      x.has_pos = c.pos;
+      x.emin = emin;
+      x.gate = gate;
+      auto go = [&](auto kern) {
+        set_smem_once(kern, c.smem);
+        kern<<<c.grid, c.nt, c.smem, st>>>(x, map);
+      };
+      if (c.nt == 256) go(k_binbuild<K, Map, 256>);
+      else if (c.nt == 512) go(k_binbuild<K, Map, 512>);
+      else go(k_binbuild<K, Map, 1024>);
     };
-    if (bc.per_sm == 2) {
-      if (bc.lb)
-        launch(k_binbuild<K, Map, 16, 2, true, false>, k_binbuild<K, Map, 16, 2, true, true>, 512);
-      else
-        launch(k_binbuild<K, Map, 16, 2, false, false>, k_binbuild<K, Map, 16, 2, false, true>, 512);
-    } else if (bc.tpb == 512) {
-      launch(k_binbuild<K, Map, 16, 1, true, false>, k_binbuild<K, Map, 16, 1, true, true>, 512);
-    } else {
-      launch(k_binbuild<K, Map, kBinNW, 1, true, false>, k_binbuild<K, Map, kBinNW, 1, true, true>, kBinNW * 32);
-    }
+    launch(bc, 0, nullptr);
+    if (bc.nt != bw.nt) launch(bw, bc.emax, wide_count);
   }
   {
     const size_t sm = big_smem_bytes(sizeof(K), 1u << p.s);
@@ -2274,8 +2342,10 @@ hg_status radix_sort_u64(uint64_t* keys, uint64_t n, uint8_t* ws, cudaStream_t s
                                        uint64_t, uint32_t*, uint8_t*, cudaStream_t, M);                   \
   template hg_status probe_binned_impl<K, M>(const ProbePlan&, uint64_t, const hg_table*, const K*,     \
                                              uint64_t, uint32_t*, uint8_t*, cudaStream_t, M);
-HG_INST(uint32_t, MurmurMap)
-HG_INST(uint64_t, MurmurMap)
+HG_INST(uint32_t, MurmurMap<true>)
+HG_INST(uint64_t, MurmurMap<true>)
+HG_INST(uint32_t, MurmurMap<false>)
+HG_INST(uint64_t, MurmurMap<false>)
 HG_INST(uint32_t, LearnedMap)
 HG_INST(uint64_t, LearnedMap)
 #undef HG_INST

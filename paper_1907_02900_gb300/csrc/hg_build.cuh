@@ -78,18 +78,12 @@ constexpr int partb_minb() {
 constexpr uint32_t kMaxItemsPerCta = 128;  // pass B work items one CTA may own
 constexpr uint32_t kMaxBinsPerCta = 256;   // bins one bin-build CTA may own
 constexpr int kPartTile = kPartNW * 32 * HG_PART_IPTQ;  // query tile: 4096 elements (smallest chunk)
-#ifndef HG_BIN_NW
-#define HG_BIN_NW 32
-#endif
-constexpr int kBinNW = HG_BIN_NW;      // warps of the bin-build kernels (1024 threads)
+constexpr int kBinNW = 32;             // warps of the oversized-bin kernels (1024 threads)
 constexpr int kBigTile = 2048;         // tile of the oversized-bin kernel
 constexpr uint32_t kBinEmaxU32 = 9216;  // largest bin built in shared memory (uint32 keys)
 constexpr uint32_t kBinEmaxU64 = 7168;  // same for uint64 keys
-constexpr uint32_t kBinSmallBucket = 32; // bucket length sorted by one thread in the bin build
 constexpr uint32_t kHugeSeg = 1u << 17;  // bins above this many edges are built by several CTAs, one per segment
 constexpr uint64_t kHugeMinN = 1ull << 22;  // ... in builds of at least this many keys
-constexpr uint32_t kBinRankBucket = 256; // longest bucket a warp ranks in registers in the bin build
-constexpr uint32_t kBinBitmapWarps = 4;  // warps sorting longer buckets with position bitmaps
 constexpr uint32_t kV1Small = 32;      // V1 fix-up: longest bucket sorted by one thread
 constexpr int kV1HeavyNW = 16;
 constexpr int kV1HeavyIPT = 8;  // V1 fix-up of long buckets: tiles of 4096
@@ -183,17 +177,17 @@ hg_status build_v1(uint64_t n, uint64_t V, const K* keys, const uint32_t* ids, u
                    K* csr_k, uint32_t* csr_i, uint8_t* ws, cudaStream_t st, Map map);
 
 // Bucket-map construction on the host.
-inline MurmurMap make_murmur(uint32_t seed, uint64_t V) {
-  MurmurMap m{};
+inline MurmurMap<true> make_murmur_pow2(uint32_t seed, uint64_t V) {  // powers of two up to 2^32
+  MurmurMap<true> m{};
   m.seed = seed;
-  if ((V & (V - 1)) == 0) {  // powers of two up to 2^32
-    m.mod.pow2 = 1;
-    m.mod.mask = (uint32_t)(V - 1);
-  } else {                   // V < 2^32
-    m.mod.pow2 = 0;
-    m.mod.d = (uint32_t)V;
-    fastmod_params((uint32_t)V, &m.mod.m, &m.mod.sh1, &m.mod.sh2);
-  }
+  m.mod.mask = (uint32_t)(V - 1);
+  return m;
+}
+inline MurmurMap<false> make_murmur(uint32_t seed, uint64_t V) {  // any other V (< 2^32)
+  MurmurMap<false> m{};
+  m.seed = seed;
+  m.mod.d = (uint32_t)V;
+  fastmod_params((uint32_t)V, &m.mod.m, &m.mod.sh1, &m.mod.sh2);
   return m;
 }
 inline LearnedMap make_learned(const void* blob, uint64_t V) {
@@ -210,7 +204,12 @@ hg_status dispatch_key_map(const hg_config* cfg, F&& f) {
     LearnedMap m = make_learned(cfg->d_model, cfg->num_buckets);
     return cfg->key_type == HG_KEY_U64 ? f(uint64_t{}, m) : f(uint32_t{}, m);
   }
-  MurmurMap m = make_murmur(cfg->seed, cfg->num_buckets);
+  const uint64_t V = cfg->num_buckets;
+  if ((V & (V - 1)) == 0) {
+    MurmurMap<true> m = make_murmur_pow2(cfg->seed, V);
+    return cfg->key_type == HG_KEY_U64 ? f(uint64_t{}, m) : f(uint32_t{}, m);
+  }
+  MurmurMap<false> m = make_murmur(cfg->seed, V);
   return cfg->key_type == HG_KEY_U64 ? f(uint64_t{}, m) : f(uint32_t{}, m);
 }
 

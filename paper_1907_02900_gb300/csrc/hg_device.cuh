@@ -52,16 +52,20 @@ __device__ __forceinline__ uint32_t murmur3(uint64_t key, uint32_t seed) {
 // l = ceil(log2 d) and m = floor(2^32 (2^l - d) / d) + 1, the quotient is
 // (t + ((h - t) >> sh1)) >> sh2 for t = high32(m h), sh1 = min(l, 1),
 // sh2 = max(l - 1, 0).  One 32-bit high multiply and one multiply-subtract.
-// Powers of two (up to 2^32) use a mask.  fastmod_params() sets it up.
+// fastmod_params() sets it up.  Powers of two (up to 2^32) use a mask; the
+// choice is a template parameter, so no kernel tests it per key.
+template <bool POW2>
 struct FastMod {
   uint32_t d, m, sh1, sh2;
-  uint32_t mask;
-  uint32_t pow2;
   __device__ __forceinline__ uint32_t operator()(uint32_t h) const {
-    if (pow2) return h & mask;
     const uint32_t t = __umulhi(m, h);
     return h - ((t + ((h - t) >> sh1)) >> sh2) * d;
   }
+};
+template <>
+struct FastMod<true> {
+  uint32_t mask;
+  __device__ __forceinline__ uint32_t operator()(uint32_t h) const { return h & mask; }
 };
 // Host side: the constants for divisor d (1 <= d < 2^32).
 inline void fastmod_params(uint32_t d, uint32_t* m, uint32_t* sh1, uint32_t* sh2) {
@@ -82,13 +86,14 @@ inline void fastmod_params(uint32_t d, uint32_t* m, uint32_t* sh1, uint32_t* sh2
 // kSkewed: the map may send most queries to a few buckets (an order-
 // preserving map does, with keys outside the fitted range); the probe then
 // merges its counts back with a balanced merge.
+template <bool POW2>
 struct MurmurMap {
   static constexpr bool kNeedsPos = false;
   static constexpr bool kSkewed = false;
   static constexpr size_t kStageBytes = 0;  // shared memory stage() can use
   uint32_t seed;
   uint32_t slab_base;
-  FastMod mod;
+  FastMod<POW2> mod;
   __device__ __forceinline__ void init() {}
   __device__ __forceinline__ void stage(uint8_t*, size_t) {}
   template <typename K>

@@ -467,8 +467,10 @@ hg_status join_materialize_impl(const hg_config* cfg, const hg_table* A, const h
                                            int64_t*, uint8_t*, cudaStream_t, M);                              \
   template hg_status join_materialize_impl<K, M>(const hg_config*, const hg_table*, const hg_table*, int64_t*, \
                                                  int64_t*, uint64_t, int64_t*, uint8_t*, cudaStream_t, M, bool);
-HG_INST(uint32_t, MurmurMap)
-HG_INST(uint64_t, MurmurMap)
+HG_INST(uint32_t, MurmurMap<true>)
+HG_INST(uint64_t, MurmurMap<true>)
+HG_INST(uint32_t, MurmurMap<false>)
+HG_INST(uint64_t, MurmurMap<false>)
 HG_INST(uint32_t, LearnedMap)
 HG_INST(uint64_t, LearnedMap)
 #undef HG_INST

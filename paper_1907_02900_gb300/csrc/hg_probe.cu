@@ -149,8 +149,10 @@ hg_status probe_launch(const K* q, uint64_t nq, const uint32_t* off, const K* ck
 #define HG_INST(K, M) \
   template hg_status probe_launch<K, M>(const K*, uint64_t, const uint32_t*, const K*, uint32_t*, uint64_t, \
                                         cudaStream_t, M, const uint32_t*);
-HG_INST(uint32_t, MurmurMap)
-HG_INST(uint64_t, MurmurMap)
+HG_INST(uint32_t, MurmurMap<true>)
+HG_INST(uint64_t, MurmurMap<true>)
+HG_INST(uint32_t, MurmurMap<false>)
+HG_INST(uint64_t, MurmurMap<false>)
 HG_INST(uint32_t, LearnedMap)
 HG_INST(uint64_t, LearnedMap)
 HG_INST(uint32_t, BatchedMap)
