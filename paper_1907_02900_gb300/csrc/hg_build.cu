@@ -247,7 +247,8 @@ struct HugeArgs {
 
 // Exclusive scan of the bin totals (one CTA); list of bins too large for the
 // shared-memory bin build (huge ones split into segments); closing CSR
-// offset offsets[V] = n; with wide_count, the number of bins of more than
+// offset offsets[V] = n; the bins' write cursors of k_partition_any's pass B
+// (cur_bin, may be null); with wide_count, the number of bins of more than
 // wide_lo and at most emax edges (the bin build's second launch).
 __global__ void __launch_bounds__(1024) k_scan_bins(const uint32_t* __restrict__ T, uint32_t nbins,
                                                     uint32_t* __restrict__ BS, uint32_t emax,
@@ -255,7 +256,8 @@ __global__ void __launch_bounds__(1024) k_scan_bins(const uint32_t* __restrict__
                                                     uint32_t* __restrict__ ovf_count,
                                                     uint32_t* __restrict__ offsets, uint64_t V,
                                                     uint32_t n_end, HugeArgs h, uint32_t* order,
-                                                    uint32_t wide_lo = 0, uint32_t* wide_count = nullptr) {
+                                                    uint32_t wide_lo = 0, uint32_t* wide_count = nullptr,
+                                                    uint32_t* __restrict__ cur_bin = nullptr) {
   // Each warp scans a contiguous range of whole 32-bin rows (lane = bin of
   // the row), so every access is coalesced: the range's sum, an exclusive
   // scan of the warp sums, then the range again from its base.
@@ -284,7 +286,11 @@ __global__ void __launch_bounds__(1024) k_scan_bins(const uint32_t* __restrict__
     const uint32_t i = r * 32u + lane;
     const uint32_t t = i < nbins ? T[i] : 0u;
     const uint32_t incl = warp_incl_scan(t);
-    if (i < nbins) BS[i] = base + incl - t;
+    if (i < nbins) {
+      const uint32_t start = base + incl - t;
+      BS[i] = start;
+      if (cur_bin) cur_bin[i] = start;
+    }
     base += __shfl_sync(kFull, incl, 31);
     if (wide_count && i < nbins && t > wide_lo && t <= emax) atomicAdd(wide_count, 1u);
     if (i >= nbins || t <= emax) continue;
@@ -331,12 +337,15 @@ struct PartArgs {
   uint64_t n, chunk;
   uint32_t G, s, sshift, nbins, nsb;
   uint32_t gg, ngroups;  // pass B: chunks per item, items per super-bin
-  const uint32_t* H;   // per (chunk, bin) exclusive column prefix
+  uint32_t piece;        // k_partition_any, pass B: tiles a CTA takes at a time
+  const uint32_t* H;   // per (chunk, bin) exclusive column prefix; row 0 (all zero) is not read: it
+                       // holds k_partition_any's cursors
   const uint32_t* C;   // per (chunk, super-bin) exclusive column prefix
   const uint32_t* CT;  // per super-bin totals
   const uint32_t* BS;  // bin starts
   uint32_t* status;
   uint32_t stage_bytes;  // shared memory after the kernel's own, for the bucket map's tables
+  uint32_t* cur_bin;   // k_partition_any, pass B: next free element of every bin
   // order mode word (null: always stable); see k_partition
   const uint32_t* order;
   // optional: per tile (tiles start at multiples of the kernel's tile size),
@@ -344,14 +353,14 @@ struct PartArgs {
   uint16_t* tile_counts;
 };
 
-// ANY: tiles ranked by shared-memory atomics, equal digits in any order
-// (tile_partition_any).  With a.order set, the build launches both variants
-// and the one that does not match the order mode written by k_scan_bins
-// returns at once: the unordered one runs only when every bin fits the
-// shared-memory bin build, which then restores the canonical order by id.
-template <typename K, typename Map, bool PASS_B, int IPT, int NW, int MINB, bool ANY>
+// The stable partition.  With a.order set, the build launches it and
+// k_partition_any, and the one that does not match the order mode written by
+// k_scan_bins returns at once: the unordered one runs only when every bin
+// fits the shared-memory bin build, which then restores the canonical order
+// by id.
+template <typename K, typename Map, bool PASS_B, int IPT, int NW, int MINB>
 __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map map) {
-  if (a.order != nullptr && ((*(volatile const uint32_t*)a.order == 0u) != ANY)) return;
+  if (a.order != nullptr && *(volatile const uint32_t*)a.order == 0u) return;
   constexpr uint32_t TILE = NW * 32 * IPT;
   constexpr uint32_t TB = TILE + 16;
   static_assert(TILE <= 65536, "tile indexes are packed into 16 bits");
@@ -477,7 +486,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map 
         const uint32_t b0 = sb << a.sshift;
         ndig = (int)min(1u << a.sshift, a.nbins - b0);
         for (int d = threadIdx.x; d < ndig; d += blockDim.x)
-          cursor[d] = a.BS[b0 + d] + a.H[(uint64_t)g * a.nbins + b0 + d];
+          cursor[d] = a.BS[b0 + d] + (g ? a.H[(uint64_t)g * a.nbins + b0 + d] : 0u);
       }
     }
     if (sync_needed) __syncthreads();  // block-uniform condition
@@ -500,23 +509,222 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map 
         dig[r] = 0;
       }
     }
-    if (ANY) {
-      if (has_ids)
-        tile_partition_any<K, IPT, NW, false>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum,
-                                              a.out_k, a.out_i, 0u);
-      else
-        tile_partition_any<K, IPT, NW, true>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum,
-                                             a.out_k, a.out_i, (uint32_t)cur.t0,
-                                             a.tile_counts ? a.tile_counts + (cur.t0 / TILE) * a.nbins : nullptr);
-    } else {
-      if (has_ids)
-        tile_partition_fast<K, IPT, NW, false>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum,
-                                               a.out_k, a.out_i, 0u);
-      else
-        tile_partition_fast<K, IPT, NW, true>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum,
-                                              a.out_k, a.out_i, (uint32_t)cur.t0);
-    }
+    if (has_ids)
+      tile_partition_fast<K, IPT, NW, false>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum, a.out_k,
+                                             a.out_i, 0u);
+    else
+      tile_partition_fast<K, IPT, NW, true>(key, val, dig, cnt, ndig, sk, sv, sd, wc, dstart, cursor, wsum, a.out_k,
+                                            a.out_i, (uint32_t)cur.t0);
     cur = nxt;
+  }
+}
+
+// Shared memory of k_partition_any (see there).
+static size_t part_any_smem(int kb, bool ids, int tile) {
+  return align_up((size_t)tile * (kb + 4 + (ids ? 1 : 0)), 16) + 4 * 256 * 4;
+}
+
+// The same passes with equal digits in any order: an element's rank in its
+// digit is the old value of a shared-memory atomic, so a tile costs one
+// atomic per element and one warp's scan of 256 counters.
+// Pass A (and the query partition): a CTA takes chunks, whose tiles follow
+// one another within each digit from the chunk's own start in it.
+// Pass B: the CTAs take equal pieces of pass A's output in turn, so all of
+// them work in a window of a few super-bins, and every tile takes its room in
+// a bin from the bin's one cursor (global atomics).  The pieces are equal
+// whatever the order or skew of the input.
+//   1. digit and rank of every element, packed in a register
+//   2. one warp: scan of the digit counts, room taken, counters cleared
+//   3. elements to their place in the digit-sorted tile in shared memory;
+//      output base of every digit (delta)
+//   4. the next tile's elements are loaded to registers, then the sorted tile
+//      is written out as runs per digit
+// IDS: the elements carry ids (else an id is the element's input position,
+// staged as its index in the tile next to its digit).
+//
+// Bound by shared-memory wavefronts: about 27 per 32 elements with the loads
+// and stores, of which the random accesses (atomic, digit start, placement)
+// make 12.  Loads go straight to registers and shared memory holds one tile
+// only, so tiles are as large as the registers allow (a run's length, TILE /
+// digits, sets how well the stores coalesce), or two CTAs share the SM.
+// 2^28 uint32 keys, against tiles staged by TMA through a double buffer:
+// pass A 1.18 -> 0.96 ms, pass B 1.41 -> 1.08, queries 1.10 -> 0.92; 2^26
+// uint64 keys under the learned map 0.63 -> 0.47, 0.78 -> 0.46, 0.49 -> 0.41.
+template <typename K, typename Map, bool PASS_B, bool IDS, int NT, int IPT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map map) {
+  if (a.order != nullptr && *(volatile const uint32_t*)a.order != 0u) return;
+  constexpr uint32_t TILE = NT * IPT;
+  static_assert(TILE <= 65536 && TILE % 16 == 0, "tile indexes are packed into 16 bits");
+  constexpr bool kPair = sizeof(K) == 4;  // key and id (or index) staged as one 8-byte element
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint8_t* sp = smem;
+  uint2* const spair = (uint2*)sp;
+  K* const sk = (K*)sp; sp += TILE * sizeof(K);
+  uint32_t* const sv = (uint32_t*)sp; sp += TILE * 4;
+  uint8_t* const sd = sp; sp += IDS ? TILE : 0;  // digits (with IDS); every size here is a multiple of 16
+  uint32_t* const tcnt = (uint32_t*)sp; sp += 256 * 4;
+  uint32_t* const dstart = (uint32_t*)sp; sp += 256 * 4;
+  uint32_t* const delta = (uint32_t*)sp; sp += 256 * 4;
+  uint32_t* const cursor = (uint32_t*)sp; sp += 256 * 4;  // pass A
+  map.init();
+  map.stage(sp, a.stage_bytes);
+  const uint32_t tid = threadIdx.x, lane = tid & 31u;
+  for (uint32_t d = tid; d < 256; d += NT) tcnt[d] = 0;
+  __syncthreads();
+  // Tile stream: the tile starts at t0 and ends at most at `end`, the end of
+  // its chunk (item) or of the part of its super-bin (item) in the CTA's
+  // piece, which ends at lim.
+  struct Ref {
+    uint32_t item, t0, end, lim;
+    bool ok;
+  };
+  const uint64_t span = PASS_B ? (uint64_t)a.piece * TILE : a.chunk;
+  auto take = [&](uint64_t c) -> Ref {  // the c-th chunk or piece
+    const uint64_t i0 = c * span;
+    const uint32_t lo = (uint32_t)i0, lim = (uint32_t)min(i0 + span, a.n);
+    if (i0 >= a.n) return Ref{0, 0, 0, 0, false};
+    if (!PASS_B) return Ref{(uint32_t)c, lo, lim, lim, true};
+    uint32_t x = 0, y = a.nsb;  // the last super-bin that starts at or before lo (of equal starts, the non-empty one)
+    while (y - x > 1) {
+      const uint32_t m = (x + y) >> 1;
+      if (__ldg(a.BS + (m << a.sshift)) <= lo) x = m;
+      else y = m;
+    }
+    return Ref{x, lo, min(__ldg(a.BS + min((x + 1) << a.sshift, a.nbins)), lim), lim, true};
+  };
+  uint64_t c_next = blockIdx.x;
+  auto advance = [&](Ref& r) {
+    r.t0 += min(r.end - r.t0, TILE);
+    if (r.t0 < r.end) return;
+    if (r.t0 < r.lim) {  // on to the piece's next super-bin that is not empty
+      do r.end = min(__ldg(a.BS + min((++r.item + 1) << a.sshift, a.nbins)), r.lim);
+      while (r.end <= r.t0);
+      return;
+    }
+    r = take(c_next += gridDim.x);
+  };
+  K key[IPT];
+  uint32_t id[IDS ? IPT : 1];
+  auto load = [&](const Ref& r) {
+    const K* const gk = a.in_k + r.t0 + tid;
+    const uint32_t* const gi = IDS ? a.in_i + r.t0 + tid : nullptr;
+    const uint32_t cnt = min(r.end - r.t0, TILE);
+    if (cnt == TILE) {
+#pragma unroll
+      for (int c = 0; c < IPT; ++c) {
+        key[c] = __ldcs(gk + c * NT);
+        if (IDS) id[IDS ? c : 0] = __ldcs(gi + c * NT);
+      }
+    } else {
+      const int left = (int)cnt - (int)tid;
+#pragma unroll
+      for (int c = 0; c < IPT; ++c) {
+        key[c] = left > c * NT ? __ldcs(gk + c * NT) : K(0);
+        if (IDS) id[IDS ? c : 0] = left > c * NT ? __ldcs(gi + c * NT) : 0u;
+      }
+    }
+  };
+  Ref cur = take(c_next);
+  if (cur.ok) load(cur);
+  const uint32_t shift = PASS_B ? a.s : a.s + a.sshift;
+  const uint32_t dmask = PASS_B ? (1u << a.sshift) - 1u : 0xffffffffu;  // pass B: bin inside the super-bin
+  uint32_t at = ~0u;  // chunk whose cursors are loaded
+  while (cur.ok) {
+    const uint32_t cnt = min(cur.end - cur.t0, TILE), t0 = cur.t0, item = cur.item;
+    const int left = (int)cnt - (int)tid;
+    if (!PASS_B && item != at) {  // first read by the scan, after a barrier
+      at = item;
+      if (tid < a.nsb) cursor[tid] = a.BS[tid << a.sshift] + a.C[(uint64_t)item * a.nsb + tid];
+    }
+    // every element through f(c): full tiles without a test per element
+    auto each = [&](auto&& f) {
+      if (cnt == TILE) {
+#pragma unroll
+        for (int c = 0; c < IPT; ++c) f(c);
+      } else {
+#pragma unroll
+        for (int c = 0; c < IPT; ++c)
+          if (left > c * NT) f(c);
+      }
+    };
+    // 1. digits and ranks
+    uint32_t dr[IPT];  // digit | rank << 8
+    each([&](int c) {
+      const uint32_t d = (map(key[c], IDS ? id[IDS ? c : 0] : t0 + tid + c * NT) >> shift) & dmask;
+      dr[c] = d | (atomicAdd(&tcnt[d], 1u) << 8);
+    });
+    __syncthreads();
+    // 2. scan of the counts (lane: 8 consecutive digits)
+    uint32_t room[PASS_B ? 8 : 1];
+    if (tid < 32) {
+      uint4* const q = reinterpret_cast<uint4*>(tcnt) + lane * 2;
+      const uint4 x = q[0], y = q[1];
+      q[0] = make_uint4(0, 0, 0, 0);
+      q[1] = make_uint4(0, 0, 0, 0);
+      const uint32_t c[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+      uint32_t sum = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) sum += c[i];
+      uint32_t run = warp_incl_scan(sum) - sum;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t d = lane * 8 + i;
+        if (PASS_B) {  // (back by the time step 3 is done)
+          room[PASS_B ? i : 0] = c[i] ? atomicAdd(a.cur_bin + (item << a.sshift) + d, c[i]) : 0u;
+        } else {
+          const uint32_t at_d = cursor[d];
+          delta[d] = at_d - run;
+          cursor[d] = at_d + c[i];
+          if (!IDS && a.tile_counts != nullptr && d < a.nbins)
+            a.tile_counts[(uint64_t)(t0 / TILE) * a.nbins + d] = (uint16_t)c[i];
+        }
+        dstart[d] = run;
+        run += c[i];
+      }
+    }
+    __syncthreads();
+    // 3. the digit-sorted tile
+    each([&](int c) {
+      const uint32_t d = dr[c] & 255u, dest = dstart[d] + (dr[c] >> 8);
+      const uint32_t v = IDS ? id[IDS ? c : 0] : (tid + c * NT) | (d << 16);
+      if (kPair) {
+        spair[dest] = make_uint2((uint32_t)key[c], v);
+      } else {
+        sk[dest] = key[c];
+        sv[dest] = v;
+      }
+      if (IDS) sd[dest] = (uint8_t)d;
+    });
+    if (PASS_B && tid < 32) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) delta[lane * 8 + i] = room[PASS_B ? i : 0] - dstart[lane * 8 + i];
+    }
+    // 4. next tile's loads, this tile's stores
+    advance(cur);
+    if (cur.ok) load(cur);
+    __syncthreads();
+    auto out = [&](uint32_t j) {
+      K k;
+      uint32_t v;
+      if (kPair) {
+        const uint2 x = spair[j];
+        k = (K)x.x;
+        v = x.y;
+      } else {
+        k = sk[j];
+        v = sv[j];
+      }
+      const uint32_t g = delta[IDS ? (uint32_t)sd[j] : v >> 16] + j;
+      a.out_k[g] = k;
+      a.out_i[g] = IDS ? v : t0 + (v & 0xffffu);
+    };
+    if (cnt == TILE) {
+#pragma unroll 4
+      for (int c = 0; c < IPT; ++c) out(tid + c * NT);
+    } else {
+      for (uint32_t j = tid; j < cnt; j += NT) out(j);
+    }
+    __syncthreads();
   }
 }
 
@@ -1353,6 +1561,18 @@ static void set_smem_once(F* kernel, size_t bytes) {
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)top);
 }
 
+// Launches k_partition_any with the tile of geometry T; the map's tables are
+// staged only where T::MINB CTAs still fit an SM.
+template <typename K, typename Map, bool PASS_B, bool IDS, typename T>
+static void partition_any(PartArgs<K> a, Map map, unsigned grid, cudaStream_t st) {
+  const DevInfo& di = dev_info();
+  const size_t own = part_any_smem(sizeof(K), IDS, T::NT * T::IPT);
+  a.stage_bytes = own + Map::kStageBytes + di.smem_reserved <= (size_t)di.smem_per_sm / T::MINB ? (uint32_t)Map::kStageBytes : 0u;
+  auto kern = k_partition_any<K, Map, PASS_B, IDS, T::NT, T::IPT, T::MINB>;
+  set_smem_once(kern, own + a.stage_bytes);
+  kern<<<grid, T::NT, own + a.stage_bytes, st>>>(a, map);
+}
+
 template <typename K, typename Map>
 hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* offsets, K* csr_k,
                    uint32_t* csr_i, uint8_t* ws, cudaStream_t st, Map map, uint32_t pos_base,
@@ -1416,7 +1636,7 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     // launch included) go to the oversized-bin kernels
     k_scan_bins<<<1, 1024, 0, st>>>(T, p.nbins, BS, emax_all, ovf, &hdr->ovf_count, offsets, p.V,
                                     pos_base + (uint32_t)p.n, h, any_order ? &hdr->order_mode : nullptr, bc.emax,
-                                    bc.nt != bw.nt ? wide_count : nullptr);
+                                    bc.nt != bw.nt ? wide_count : nullptr, any_order ? H : nullptr);
   }
 
   PartArgs<K> pa{};
@@ -1438,28 +1658,23 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   pa.C = C;
   pa.CT = CT;
   pa.BS = BS;
+  pa.cur_bin = H;  // chunk 0's row
   pa.status = status;
   {
     pa.order = any_order ? &hdr->order_mode : nullptr;
-    // the map's tables are staged only where they fit next to the tile
-    auto launch = [&](auto kern, int ipt) {
-      PartArgs<K> x = pa;
-      const size_t own = part_smem_bytes(sizeof(K), ids != nullptr, ipt, false, kPartNW);
-      x.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
-      set_smem_once(kern, own + x.stage_bytes);
-      kern<<<p.G, kPartNW * 32, own + x.stage_bytes, st>>>(x, map);
-    };
     HG_TRACE("k_partition_A", st);
-    // (a tile of carried ids takes the stable variant's tile size: the
-    // larger one leaves no room for staging the ids)
-    if (any_order && ids == nullptr)
-      launch(k_partition<K, Map, false, part_ipt_keys<K, true>(), kPartNW, part_minb_keys<K, true>(), true>,
-             part_ipt_keys<K, true>());
-    else if (any_order)
-      launch(k_partition<K, Map, false, part_ipt_keys<K, false>(), kPartNW, part_minb_keys<K, false>(), true>,
-             part_ipt_keys<K, false>());
-    launch(k_partition<K, Map, false, part_ipt_keys<K, false>(), kPartNW, part_minb_keys<K, false>(), false>,
-           part_ipt_keys<K, false>());
+    if (any_order) {
+      if (ids == nullptr) partition_any<K, Map, false, false, PartA<K>>(pa, map, p.G, st);
+      else partition_any<K, Map, false, true, PartB<K>>(pa, map, p.G, st);
+    }
+    // the map's tables are staged only where they fit next to the tile
+    constexpr int ipt = part_ipt_keys<K>();
+    auto kern = k_partition<K, Map, false, ipt, kPartNW, part_minb_keys<K>()>;
+    PartArgs<K> x = pa;
+    const size_t own = part_smem_bytes(sizeof(K), ids != nullptr, ipt, false, kPartNW);
+    x.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
+    set_smem_once(kern, own + x.stage_bytes);
+    kern<<<p.G, kPartNW * 32, own + x.stage_bytes, st>>>(x, map);
   }
   if (two) {
     PartArgs<K> pb = pa;
@@ -1473,18 +1688,23 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     pb.gg = (uint32_t)std::min<uint64_t>(p.G, std::max<uint64_t>(1, 32768 / per_chunk_sb));
     pb.ngroups = (p.G + pb.gg - 1) / pb.gg;
     const uint64_t items = (uint64_t)p.nsb * pb.ngroups;
-    auto launch = [&](auto kern, int nw) {
-      const size_t sm = part_smem_bytes(sizeof(K), true, kPartIPTB, true, nw);
-      set_smem_once(kern, sm);
-      int per_sm = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nw * 32, sm);
-      unsigned grid = (unsigned)std::min<uint64_t>(items, (uint64_t)std::max(1, per_sm) * di.sms);
-      grid = (unsigned)std::max<uint64_t>(grid, (items + kMaxItemsPerCta - 1) / kMaxItemsPerCta);
-      kern<<<grid, nw * 32, sm, st>>>(pb, map);
-    };
     HG_TRACE("k_partition_B", st);
-    if (any_order) launch(k_partition<K, Map, true, kPartIPTB, partb_nw<true>(), partb_minb<true>(), true>, partb_nw<true>());
-    launch(k_partition<K, Map, true, kPartIPTB, partb_nw<false>(), partb_minb<false>(), false>, partb_nw<false>());
+    if (any_order) {
+      // four pieces or more per resident CTA, of at most kPartPiece tiles
+      constexpr uint64_t tile = (uint64_t)PartB<K>::NT * PartB<K>::IPT;
+      const uint64_t resident = (uint64_t)PartB<K>::MINB * di.sms, tiles = (p.n + tile - 1) / tile;
+      pb.piece = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kPartPiece, tiles / (4 * resident)));
+      const uint64_t pieces = (tiles + pb.piece - 1) / pb.piece;
+      partition_any<K, Map, true, true, PartB<K>>(pb, map, (unsigned)std::min(pieces, resident), st);
+    }
+    auto kern = k_partition<K, Map, true, kPartIPTB, kPartNWB, kPartMinBlocksB>;
+    const size_t sm = part_smem_bytes(sizeof(K), true, kPartIPTB, true, kPartNWB);
+    set_smem_once(kern, sm);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPartNWB * 32, sm);
+    unsigned grid = (unsigned)std::min<uint64_t>(items, (uint64_t)std::max(1, per_sm) * di.sms);
+    grid = (unsigned)std::max<uint64_t>(grid, (items + kMaxItemsPerCta - 1) / kMaxItemsPerCta);
+    kern<<<grid, kPartNWB * 32, sm, st>>>(pb, map);
   }
   // A partition that could not be launched (say, a tile geometry built in at
   // compile time that needs more shared memory than a CTA may have) left the
@@ -1665,8 +1885,8 @@ hg_status build_slabs(const hg_config* cfg, const SlabPlan& p, const K* keys, co
     pa.BS = BS;
     pa.status = &hdr->status;
     pa.order = nullptr;
-    constexpr int ipt = part_ipt_keys<K, false>();
-    auto kern = k_partition<K, Map, false, ipt, kPartNW, part_minb_keys<K, false>(), false>;
+    constexpr int ipt = part_ipt_keys<K>();
+    auto kern = k_partition<K, Map, false, ipt, kPartNW, part_minb_keys<K>()>;
     const size_t own = part_smem_bytes(sizeof(K), ids != nullptr, ipt, false, kPartNW);
     pa.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
     set_smem_once(kern, own + pa.stage_bytes);
@@ -1944,22 +2164,22 @@ __global__ void __launch_bounds__(kUnpermuteThreads) k_unpermute_bal(
   }
 }
 
-// Queries are grouped by a partition that ranks each tile in any order (its
-// tiles are whole blocks of kQueryBlock positions or the end of the
-// queries).  A group's positions are therefore ascending from block to
+// Queries are grouped by a partition that ranks each tile in any order
+// (whole tiles make up a block of kQueryBlock positions, but for the end of
+// the queries).  A group's positions are therefore ascending from block to
 // block, though not inside a block's run, and the merge works in output
 // tiles made of whole blocks: within a group, every query of an earlier
 // output tile precedes every query of a later one, which is all its
 // cursors need.
-constexpr uint64_t kQueryBlock = 4096;
-static_assert(kQueryBlock % (kPartNW * 32 * part_ipt_queries<uint32_t>()) == 0 &&
-                  kQueryBlock % (kPartNW * 32 * part_ipt_queries<uint64_t>()) == 0 && kUnpermuteTile % kQueryBlock == 0,
+constexpr uint64_t kQueryBlock = 8192;
+static_assert(kQueryBlock % (PartQ<uint32_t>::NT * PartQ<uint32_t>::IPT) == 0 &&
+                  kQueryBlock % (PartQ<uint64_t>::NT * PartQ<uint64_t>::IPT) == 0 && kUnpermuteTile % kQueryBlock == 0,
               "query blocks are whole partition tiles; merge tiles are whole blocks");
 
 // Elements per tile of the query partition (whole tiles per query block).
 static uint32_t query_tile(int kb) {
-  return kb == 8 ? (uint32_t)(kPartNW * 32 * part_ipt_queries<uint64_t>())
-                 : (uint32_t)(kPartNW * 32 * part_ipt_queries<uint32_t>());
+  return kb == 8 ? (uint32_t)(PartQ<uint64_t>::NT * PartQ<uint64_t>::IPT)
+                 : (uint32_t)(PartQ<uint32_t>::NT * PartQ<uint32_t>::IPT);
 }
 
 #ifndef HG_PROBE_GROUP_BITS
@@ -1980,7 +2200,7 @@ bool make_probe_plan(const hg_config* cfg, uint64_t table_n, uint64_t q, ProbePl
   p->ng = (uint32_t)(((V - 1) >> sg) + 1);
   if (p->ng > 256) return false;
   const int sms = std::max(di.sms, 1);
-  // chunks are whole 4096-query blocks, so every partition tile lies in one
+  // chunks are whole query blocks, so every partition tile lies in one
   // block (the merge below relies on it)
   uint64_t chunk = std::max<uint64_t>(kPartTile, (q + 2 * sms - 1) / (2 * sms));
   chunk = (chunk + kQueryBlock - 1) / kQueryBlock * kQueryBlock;
@@ -2051,13 +2271,8 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
   pa.status = &hdr->status;
   pa.tile_counts = Map::kSkewed ? (uint16_t*)(ws + p.o_tc) : nullptr;
   {
-    const size_t own = part_smem_bytes(sizeof(K), false, part_ipt_queries<K>(), false, kPartNW);
-    pa.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
-    const size_t sm = own + pa.stage_bytes;
-    auto kern = k_partition<K, Map, false, part_ipt_queries<K>(), kPartNW, kPartMinBlocksQ, true>;
-    set_smem_once(kern, sm);
     HG_TRACE("k_partition_Q", st);
-    kern<<<p.G, kPartNW * 32, sm, st>>>(pa, map);
+    partition_any<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
   }
   // the probe and the merge index by the grouped positions: none may run on
   // a query partition that was not launched
@@ -2066,7 +2281,7 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
                                       Map::kNeedsPos ? qi : nullptr);
   if (rc != HG_OK) return rc;
   {
-    // every CTA merges a span of at least 4096 outputs (in tiles of up to
+    // every CTA merges a span of at least one block of outputs (in tiles of up to
     // kUnpermuteTile), so small batches still spread over the SMs
     const uint64_t blocks = (q + kQueryBlock - 1) / kQueryBlock;
     const uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(blocks, (uint64_t)2 * di.sms));
@@ -2176,12 +2391,8 @@ hg_status probe_slabs(const hg_config* cfg, const SlabProbePlan& p, const hg_tab
     pa.BS = GS;
     pa.status = &hdr->status;
     pa.tile_counts = Map::kSkewed ? (uint16_t*)(ws + p.o_tc) : nullptr;
-    const size_t own = part_smem_bytes(sizeof(K), false, part_ipt_queries<K>(), false, kPartNW);
-    pa.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
-    auto kern = k_partition<K, Map, false, part_ipt_queries<K>(), kPartNW, kPartMinBlocksQ, true>;
-    set_smem_once(kern, own + pa.stage_bytes);
     HG_TRACE("k_partition_Q", st);
-    kern<<<p.G, kPartNW * 32, own + pa.stage_bytes, st>>>(pa, map);
+    partition_any<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
   }
   if (cudaPeekAtLastError() != cudaSuccess) return last_launch_status();  // partition not launched
   // 2. slab query counts to the host, then the binned probe of every slab
@@ -2284,8 +2495,8 @@ hg_status radix_sort_u64(uint64_t* keys, uint64_t n, uint8_t* ws, cudaStream_t s
   uint32_t* ids = (uint32_t*)(ws + o[6]);
   uint64_t* src = keys;
   uint64_t* dst = tmp;
-  const size_t psm = part_smem_bytes(8, false, part_ipt_queries<uint64_t>(), false, kPartNW);
-  auto kp = k_partition<uint64_t, RadixByteMap, false, part_ipt_queries<uint64_t>(), kPartNW, kPartMinBlocksQ, false>;
+  const size_t psm = part_smem_bytes(8, false, part_ipt_keys<uint64_t>(), false, kPartNW);
+  auto kp = k_partition<uint64_t, RadixByteMap, false, part_ipt_keys<uint64_t>(), kPartNW, part_minb_keys<uint64_t>()>;
   set_smem_once(kp, psm);
   auto kh = k_hist<uint64_t, RadixByteMap>;
   const size_t hsm = hist_stage_offset(256);

@@ -8,76 +8,39 @@ namespace hg {
 constexpr int kHistThreads = 1024;
 constexpr uint32_t kMaxBinsLog2 = 15;  // bins counted in one shared-memory histogram
 constexpr uint32_t kMaxBinShift = 15;  // buckets per bin <= 2^15 (u16 local index, 128 KB cursors)
-// Partition geometry (compile-time; the defaults are the tuned values).
-// Pass A (keys) and the query partition share a kernel but not their tiles:
-// the query tiles must be powers of two (whole blocks of the probe's merge).
-// The tile ranking in any order (k_partition ANY) and the stable ranking
-// are tuned separately: they cost different registers and instructions.
-#ifndef HG_PART_NW
-#define HG_PART_NW 16
-#endif
-#ifndef HG_PART_IPT
-#define HG_PART_IPT 20  // pass A, 4-byte keys, any order: tiles of 10240, one CTA per SM
-#endif
-#ifndef HG_PART_MINB
-#define HG_PART_MINB 1
-#endif
-#ifndef HG_PART_IPTS
-#define HG_PART_IPTS 16  // pass A, 4-byte keys, stable: tiles of 8192, one CTA per SM
-#endif
-#ifndef HG_PART_MINBS
-#define HG_PART_MINBS 1
-#endif
-#ifndef HG_PART_IPTQ
-#define HG_PART_IPTQ 8  // query partition (and the sample sort), 4-byte keys: tiles of 4096
-#endif
-#ifndef HG_PART_MINBQ
-#define HG_PART_MINBQ 2
-#endif
-#ifndef HG_PART_IPT64
-#define HG_PART_IPT64 4  // 8-byte keys, everywhere: tiles of 2048, two CTAs per SM
-#endif
-#ifndef HG_PART_IPTB
-#define HG_PART_IPTB 6  // pass B items per thread
-#endif
-#ifndef HG_PARTB_NW
-#define HG_PARTB_NW 16  // pass B, any order: 512-thread CTAs, two per SM
-#endif
-#ifndef HG_PARTB_MINB
-#define HG_PARTB_MINB 2
-#endif
-#ifndef HG_PARTB_NWS
-#define HG_PARTB_NWS 8  // pass B, stable: 256-thread CTAs, up to four per SM
-#endif
-#ifndef HG_PARTB_MINBS
-#define HG_PARTB_MINBS 4
-#endif
-constexpr int kPartNW = HG_PART_NW;  // warps of the pass A / query partition CTAs
-template <typename K, bool ANY>
-constexpr int part_ipt_keys() {  // pass A items per thread
-  return sizeof(K) == 8 ? HG_PART_IPT64 : ANY ? HG_PART_IPT : HG_PART_IPTS;
-}
-template <typename K, bool ANY>
-constexpr int part_minb_keys() {
-  return sizeof(K) == 8 ? 2 : ANY ? HG_PART_MINB : HG_PART_MINBS;
+// Partition geometry.  Stable passes: warps per CTA, items per thread,
+// resident CTAs per SM.
+constexpr int kPartNW = 16;
+template <typename K>
+constexpr int part_ipt_keys() {  // pass A: tiles of 8192 4-byte or 2048 8-byte keys
+  return sizeof(K) == 8 ? 4 : 16;
 }
 template <typename K>
-constexpr int part_ipt_queries() {  // query partition items per thread
-  return sizeof(K) == 8 ? HG_PART_IPT64 : HG_PART_IPTQ;
+constexpr int part_minb_keys() {
+  return sizeof(K) == 8 ? 2 : 1;
 }
-constexpr int kPartMinBlocksQ = HG_PART_MINBQ;
-constexpr int kPartIPTB = HG_PART_IPTB;
-template <bool ANY>
-constexpr int partb_nw() {
-  return ANY ? HG_PARTB_NW : HG_PARTB_NWS;
-}
-template <bool ANY>
-constexpr int partb_minb() {
-  return ANY ? HG_PARTB_MINB : HG_PARTB_MINBS;
-}
+constexpr int kPartIPTB = 6;  // pass B: 256-thread CTAs, up to four per SM
+constexpr int kPartNWB = 8;
+constexpr int kPartMinBlocksB = 4;
+// Passes in any order: threads per CTA, items per thread, resident CTAs per
+// SM, by measured sweeps (ms, build and probe of 2^28 uint32 keys, then of
+// 2^26 uint64 keys under the learned map).
+template <typename K>
+struct PartA {  // input positions as ids: tiles of 12288; 20 items 1.02, 28 items 0.98, 2 CTAs of 20 items 1.31 / of 5632
+  static constexpr int NT = 512, IPT = sizeof(K) == 8 ? 11 : 24, MINB = sizeof(K) == 8 ? 2 : 1;  // 0.96 / 0.47
+};
+template <typename K>
+struct PartB {  // elements with ids: tiles of 4608 / 4096; 12 items 1.23, 16 items with one CTA 1.24 / 12 items 0.55
+  static constexpr int NT = 512, IPT = sizeof(K) == 8 ? 8 : 9, MINB = 2;  // 1.11 / 0.46
+};
+template <typename K>
+struct PartQ {  // queries: tiles of 8192 / 4096 (they divide kQueryBlock); two CTAs of 4096 1.07 / one of 8192 0.51
+  static constexpr int NT = 512, IPT = sizeof(K) == 8 ? 8 : 16, MINB = sizeof(K) == 8 ? 2 : 1;  // 0.92 / 0.41
+};
+constexpr uint32_t kPartPiece = 8;  // pass B: most tiles a CTA takes at a time (1: 1.19 ms, 4: 1.11, 8: 1.08)
 constexpr uint32_t kMaxItemsPerCta = 128;  // pass B work items one CTA may own
 constexpr uint32_t kMaxBinsPerCta = 256;   // bins one bin-build CTA may own
-constexpr int kPartTile = kPartNW * 32 * HG_PART_IPTQ;  // query tile: 4096 elements (smallest chunk)
+constexpr int kPartTile = 4096;  // smallest chunk of keys
 constexpr int kBinNW = 32;             // warps of the oversized-bin kernels (1024 threads)
 constexpr int kBigTile = 2048;         // tile of the oversized-bin kernel
 constexpr uint32_t kBinEmaxU32 = 9216;  // largest bin built in shared memory (uint32 keys)
