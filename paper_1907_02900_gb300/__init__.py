@@ -260,7 +260,16 @@ def probe_into(table: Table, queries, counts, stream=None):
     _check(rc, "hg_probe")
 
 
-BINNED_PROBE_MIN_QUERIES = 1 << 20
+def _binning_pays(table: Table, q: int) -> bool:
+    """Whether the binned probe of q queries is the faster one.  The direct probe is bound by random accesses, which
+    L2 (129 MB) serves at several times the rate of DRAM; the binned one adds three passes over the queries.  Direct
+    against binned, us, at load 1: uint32 keys, a 64 MB table 531 / 1013 at 2^26 queries; 128 MB 278 / 303 at 2^24 and
+    1089 / 1019 at 2^26; 256 MB 127 / 133 at 2^22 and 483 / 304 at 2^24; 2 GB 204 / 235 at 2^22 and 796 / 650 at
+    2^24; uint64 keys, 96 MB 711 / 1221 at 2^26; 192 MB 384 / 349 at 2^24."""
+    mb = (4 * table.num_buckets + table.keys.numel() * table.keys.element_size()) >> 20
+    if mb <= 96:
+        return False
+    return q > (1 << 25 if mb <= 160 else 1 << 24 if mb <= 224 else 1 << 22)
 
 
 def probe_workspace_size(table: Table, q: int) -> int:
@@ -277,14 +286,16 @@ def probe_binned_into(table: Table, queries, counts, ws, stream=None):
 
 def probe(table: Table, queries, stream=None, binned: bool | None = None, ws=None):
     """uint32 count of build keys equal to each query (HashGraph-Probe-Standard
-    semantics).  binned=None picks the binned probe for large batches."""
+    semantics).  binned=None picks the faster of the direct and the binned probe."""
     torch = _torch()
     _require_cuda(queries, "queries")
     if _key_type_of(queries) != table.cfg.key_type:
         raise TypeError("query key type differs from the table's")
     counts = torch.empty(queries.numel(), dtype=torch.uint32, device=queries.device)
     if binned is None:
-        binned = queries.numel() >= BINNED_PROBE_MIN_QUERIES
+        binned = _binning_pays(table, queries.numel())
+        if not binned and queries.numel() >= 1 << 20 and queries.data_ptr() % 16:
+            raise HGError(1, "hg_probe")  # large batches are 16-byte aligned, whichever probe takes them
     if binned:
         need = probe_workspace_size(table, queries.numel())
         if need == 0:
