@@ -266,6 +266,8 @@ def _binning_pays(table: Table, q: int) -> bool:
     against binned, us, at load 1: uint32 keys, a 64 MB table 531 / 1013 at 2^26 queries; 128 MB 278 / 303 at 2^24 and
     1089 / 1019 at 2^26; 256 MB 127 / 133 at 2^22 and 483 / 304 at 2^24; 2 GB 204 / 235 at 2^22 and 796 / 650 at
     2^24; uint64 keys, 96 MB 711 / 1221 at 2^26; 192 MB 384 / 349 at 2^24."""
+    if q <= 1 << 22:
+        return False
     mb = (4 * table.num_buckets + table.keys.numel() * table.keys.element_size()) >> 20
     if mb <= 96:
         return False
@@ -293,8 +295,9 @@ def probe(table: Table, queries, stream=None, binned: bool | None = None, ws=Non
         raise TypeError("query key type differs from the table's")
     counts = torch.empty(queries.numel(), dtype=torch.uint32, device=queries.device)
     if binned is None:
-        binned = _binning_pays(table, queries.numel())
-        if not binned and queries.numel() >= 1 << 20 and queries.data_ptr() % 16:
+        q = queries.numel()
+        binned = _binning_pays(table, q)
+        if not binned and q >= 1 << 20 and queries.data_ptr() % 16:
             raise HGError(1, "hg_probe")  # large batches are 16-byte aligned, whichever probe takes them
     if binned:
         need = probe_workspace_size(table, queries.numel())

@@ -520,13 +520,13 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map 
 }
 
 // Shared memory of k_partition_any (see there).
-static size_t part_any_smem(int kb, bool ids, int tile) {
-  return align_up((size_t)tile * (kb + 4 + (ids ? 1 : 0)), 16) + 4 * 256 * 4;
+static size_t part_any_smem(int kb, bool ids, int tile, int digits) {
+  return align_up((size_t)tile * (kb + 4 + (ids ? 1 : 0)), 16) + 4 * (size_t)digits * 4;
 }
 
 // The same passes with equal digits in any order: an element's rank in its
 // digit is the old value of a shared-memory atomic, so a tile costs one
-// atomic per element and one warp's scan of 256 counters.
+// atomic per element and one warp's scan of the DIG counters (256 or 512).
 // Pass A (and the query partition): a CTA takes chunks, whose tiles follow
 // one another within each digit from the chunk's own start in it.
 // Pass B: the CTAs take equal pieces of pass A's output in turn, so all of
@@ -550,11 +550,13 @@ static size_t part_any_smem(int kb, bool ids, int tile) {
 // 2^28 uint32 keys, against tiles staged by TMA through a double buffer:
 // pass A 1.18 -> 0.96 ms, pass B 1.41 -> 1.08, queries 1.10 -> 0.92; 2^26
 // uint64 keys under the learned map 0.63 -> 0.47, 0.78 -> 0.46, 0.49 -> 0.41.
-template <typename K, typename Map, bool PASS_B, bool IDS, int NT, int IPT, int MINB>
+template <typename K, typename Map, bool PASS_B, bool IDS, int DIG, int NT, int IPT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map map) {
   if (a.order != nullptr && *(volatile const uint32_t*)a.order != 0u) return;
   constexpr uint32_t TILE = NT * IPT;
   static_assert(TILE <= 65536 && TILE % 16 == 0, "tile indexes are packed into 16 bits");
+  static_assert(DIG == 256 || (DIG == 512 && !IDS && NT >= 512), "digits fit their packings");
+  constexpr int DBITS = DIG == 512 ? 9 : 8, PER = DIG / 32;
   constexpr bool kPair = sizeof(K) == 4;  // key and id (or index) staged as one 8-byte element
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t* sp = smem;
@@ -562,14 +564,14 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
   K* const sk = (K*)sp; sp += TILE * sizeof(K);
   uint32_t* const sv = (uint32_t*)sp; sp += TILE * 4;
   uint8_t* const sd = sp; sp += IDS ? TILE : 0;  // digits (with IDS); every size here is a multiple of 16
-  uint32_t* const tcnt = (uint32_t*)sp; sp += 256 * 4;
-  uint32_t* const dstart = (uint32_t*)sp; sp += 256 * 4;
-  uint32_t* const delta = (uint32_t*)sp; sp += 256 * 4;
-  uint32_t* const cursor = (uint32_t*)sp; sp += 256 * 4;  // pass A
+  uint32_t* const tcnt = (uint32_t*)sp; sp += DIG * 4;
+  uint32_t* const dstart = (uint32_t*)sp; sp += DIG * 4;
+  uint32_t* const delta = (uint32_t*)sp; sp += DIG * 4;
+  uint32_t* const cursor = (uint32_t*)sp; sp += DIG * 4;  // pass A
   map.init();
   map.stage(sp, a.stage_bytes);
   const uint32_t tid = threadIdx.x, lane = tid & 31u;
-  for (uint32_t d = tid; d < 256; d += NT) tcnt[d] = 0;
+  for (uint32_t d = tid; d < DIG; d += NT) tcnt[d] = 0;
   __syncthreads();
   // Tile stream: the tile starts at t0 and ends at most at `end`, the end of
   // its chunk (item) or of the part of its super-bin (item) in the CTA's
@@ -648,27 +650,32 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
       }
     };
     // 1. digits and ranks
-    uint32_t dr[IPT];  // digit | rank << 8
+    uint32_t dr[IPT];  // digit | rank << DBITS
     each([&](int c) {
       const uint32_t d = (map(key[c], IDS ? id[IDS ? c : 0] : t0 + tid + c * NT) >> shift) & dmask;
-      dr[c] = d | (atomicAdd(&tcnt[d], 1u) << 8);
+      dr[c] = d | (atomicAdd(&tcnt[d], 1u) << DBITS);
     });
     __syncthreads();
-    // 2. scan of the counts (lane: 8 consecutive digits)
-    uint32_t room[PASS_B ? 8 : 1];
+    // 2. scan of the counts (lane: PER consecutive digits)
+    uint32_t room[PASS_B ? PER : 1];
     if (tid < 32) {
-      uint4* const q = reinterpret_cast<uint4*>(tcnt) + lane * 2;
-      const uint4 x = q[0], y = q[1];
-      q[0] = make_uint4(0, 0, 0, 0);
-      q[1] = make_uint4(0, 0, 0, 0);
-      const uint32_t c[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+      uint32_t c[PER];
       uint32_t sum = 0;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) sum += c[i];
+      for (int i = 0; i < PER; i += 4) {
+        uint4* const q = reinterpret_cast<uint4*>(tcnt + lane * PER + i);
+        const uint4 x = *q;
+        *q = make_uint4(0, 0, 0, 0);
+        c[i] = x.x;
+        c[i + 1] = x.y;
+        c[i + 2] = x.z;
+        c[i + 3] = x.w;
+        sum += x.x + x.y + x.z + x.w;
+      }
       uint32_t run = warp_incl_scan(sum) - sum;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint32_t d = lane * 8 + i;
+      for (int i = 0; i < PER; ++i) {
+        const uint32_t d = lane * PER + i;
         if (PASS_B) {  // (back by the time step 3 is done)
           room[PASS_B ? i : 0] = c[i] ? atomicAdd(a.cur_bin + (item << a.sshift) + d, c[i]) : 0u;
         } else {
@@ -685,7 +692,7 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
     __syncthreads();
     // 3. the digit-sorted tile
     each([&](int c) {
-      const uint32_t d = dr[c] & 255u, dest = dstart[d] + (dr[c] >> 8);
+      const uint32_t d = dr[c] & (DIG - 1u), dest = dstart[d] + (dr[c] >> DBITS);
       const uint32_t v = IDS ? id[IDS ? c : 0] : (tid + c * NT) | (d << 16);
       if (kPair) {
         spair[dest] = make_uint2((uint32_t)key[c], v);
@@ -697,7 +704,7 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
     });
     if (PASS_B && tid < 32) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) delta[lane * 8 + i] = room[PASS_B ? i : 0] - dstart[lane * 8 + i];
+      for (int i = 0; i < PER; ++i) delta[lane * PER + i] = room[PASS_B ? i : 0] - dstart[lane * PER + i];
     }
     // 4. next tile's loads, this tile's stores
     advance(cur);
@@ -725,6 +732,46 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
       for (uint32_t j = tid; j < cnt; j += NT) out(j);
     }
     __syncthreads();
+  }
+}
+
+// Bin totals after pass A, for builds of more bins than one shared-memory
+// histogram of the whole input holds: the CTAs take equal pieces of pass A's
+// output in turn and count a piece's bins super-bin by super-bin (up to 256
+// bins each), then add the counts to T (zeroed before).
+constexpr uint32_t kLatePiece = 32768;
+template <typename K, typename Map>
+__global__ void __launch_bounds__(512) k_hist_late(PartArgs<K> a, uint32_t* __restrict__ T, Map map) {
+  __shared__ uint32_t hist[256];
+  map.init();
+  const uint32_t dmask = (1u << a.sshift) - 1u;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * kLatePiece; i0 < a.n; i0 += (uint64_t)gridDim.x * kLatePiece) {
+    const uint32_t lim = (uint32_t)min(i0 + kLatePiece, a.n);
+    uint32_t x = 0, y = a.nsb;  // the last super-bin that starts at or before i0
+    while (y - x > 1) {
+      const uint32_t m = (x + y) >> 1;
+      if (__ldg(a.BS + m) <= (uint32_t)i0) x = m;
+      else y = m;
+    }
+    for (uint32_t t0 = (uint32_t)i0; t0 < lim; ++x) {
+      const uint32_t end = min(__ldg(a.BS + x + 1), lim);
+      if (end <= t0) continue;  // (block-uniform) an empty super-bin
+      if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+      __syncthreads();
+      uint32_t j = t0 + threadIdx.x;
+      for (; j < end && end - j > 7 * 512; j += 8 * 512) {  // eight loads in flight
+        K k[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) k[u] = __ldcs(a.in_k + j + u * 512);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) atomicAdd(&hist[(map(k[u]) >> a.s) & dmask], 1u);
+      }
+      for (; j < end; j += 512) atomicAdd(&hist[(map(__ldcs(a.in_k + j)) >> a.s) & dmask], 1u);
+      __syncthreads();
+      if (threadIdx.x <= dmask && hist[threadIdx.x] != 0) atomicAdd(T + ((uint64_t)x << a.sshift) + threadIdx.x, hist[threadIdx.x]);
+      __syncthreads();
+      t0 = end;
+    }
   }
 }
 
@@ -1223,6 +1270,15 @@ static BinCfg bin_config(const Plan& p, bool by_id) {
   return bin_config_for<K>(p, 1024, true);
 }
 
+// The two launches: bins up to first->emax, and larger ones up to
+// second->emax (no such launch where both have 1024 threads).
+template <typename K>
+static void bin_configs(const Plan& p, bool by_id, BinCfg* first, BinCfg* second) {
+  *first = bin_config<K>(p, by_id);
+  *second = bin_config_for<K>(p, 1024, true);
+  first->emax = std::min(first->emax, second->emax);
+}
+
 // Streams edges [start, start + len) of a bin in tiles of kBigTile, sorts
 // every tile stably by local bucket and appends each run at its bucket's
 // cursor (cur: absolute CSR positions of the bin's nb buckets, advanced).
@@ -1563,14 +1619,44 @@ static void set_smem_once(F* kernel, size_t bytes) {
 
 // Launches k_partition_any with the tile of geometry T; the map's tables are
 // staged only where T::MINB CTAs still fit an SM.
-template <typename K, typename Map, bool PASS_B, bool IDS, typename T>
+template <typename K, typename Map, bool PASS_B, bool IDS, typename T, int DIG = 256>
 static void partition_any(PartArgs<K> a, Map map, unsigned grid, cudaStream_t st) {
   const DevInfo& di = dev_info();
-  const size_t own = part_any_smem(sizeof(K), IDS, T::NT * T::IPT);
+  const size_t own = part_any_smem(sizeof(K), IDS, T::NT * T::IPT, DIG);
   a.stage_bytes = own + Map::kStageBytes + di.smem_reserved <= (size_t)di.smem_per_sm / T::MINB ? (uint32_t)Map::kStageBytes : 0u;
-  auto kern = k_partition_any<K, Map, PASS_B, IDS, T::NT, T::IPT, T::MINB>;
+  auto kern = k_partition_any<K, Map, PASS_B, IDS, DIG, T::NT, T::IPT, T::MINB>;
   set_smem_once(kern, own + a.stage_bytes);
   kern<<<grid, T::NT, own + a.stage_bytes, st>>>(a, map);
+}
+
+// Pass B in any order: four pieces or more per resident CTA, of at most
+// kPartPiece tiles.
+template <typename K, typename Map>
+static void partition_b_any(PartArgs<K> a, Map map, cudaStream_t st) {
+  constexpr uint64_t tile = (uint64_t)PartB<K>::NT * PartB<K>::IPT;
+  const uint64_t resident = (uint64_t)PartB<K>::MINB * dev_info().sms, tiles = (a.n + tile - 1) / tile;
+  a.piece = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kPartPiece, tiles / (4 * resident)));
+  const uint64_t pieces = (tiles + a.piece - 1) / a.piece;
+  partition_any<K, Map, true, true, PartB<K>>(a, map, (unsigned)std::min(pieces, resident), st);
+}
+
+// One bin-build launch (k_binbuild): bins of more than emin edges (0: all) up
+// to the configuration's largest.
+template <typename K, typename Map>
+static void binbuild_launch(BinArgs<K> a, Map map, const BinCfg& c, uint32_t emin, const uint32_t* gate,
+                            cudaStream_t st) {
+  a.emax = c.emax;
+  a.list = c.list;
+  a.has_pos = c.pos;
+  a.emin = emin;
+  a.gate = gate;
+  auto go = [&](auto kern) {
+    set_smem_once(kern, c.smem);
+    kern<<<c.grid, c.nt, c.smem, st>>>(a, map);
+  };
+  if (c.nt == 256) go(k_binbuild<K, Map, 256>);
+  else if (c.nt == 512) go(k_binbuild<K, Map, 512>);
+  else go(k_binbuild<K, Map, 1024>);
 }
 
 template <typename K, typename Map>
@@ -1615,9 +1701,8 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   // Both variants of each such kernel are launched; the one that does not
   // match the order mode returns at once.
   const bool any_order = ids == nullptr || positional_ids;
-  BinCfg bc = bin_config<K>(p, any_order);
-  const BinCfg bw = bin_config_for<K>(p, 1024, true);  // bins larger than bc.emax
-  bc.emax = std::min(bc.emax, bw.emax);
+  BinCfg bc, bw;
+  bin_configs<K>(p, any_order, &bc, &bw);
   const uint32_t emax_all = bw.emax;
   // bins for the bin build's second launch, counted by k_scan_bins
   uint32_t* const wide_count = (uint32_t*)&hdr->counters[7];
@@ -1689,14 +1774,7 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     pb.ngroups = (p.G + pb.gg - 1) / pb.gg;
     const uint64_t items = (uint64_t)p.nsb * pb.ngroups;
     HG_TRACE("k_partition_B", st);
-    if (any_order) {
-      // four pieces or more per resident CTA, of at most kPartPiece tiles
-      constexpr uint64_t tile = (uint64_t)PartB<K>::NT * PartB<K>::IPT;
-      const uint64_t resident = (uint64_t)PartB<K>::MINB * di.sms, tiles = (p.n + tile - 1) / tile;
-      pb.piece = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kPartPiece, tiles / (4 * resident)));
-      const uint64_t pieces = (tiles + pb.piece - 1) / pb.piece;
-      partition_any<K, Map, true, true, PartB<K>>(pb, map, (unsigned)std::min(pieces, resident), st);
-    }
+    if (any_order) partition_b_any<K, Map>(pb, map, st);
     auto kern = k_partition<K, Map, true, kPartIPTB, kPartNWB, kPartMinBlocksB>;
     const size_t sm = part_smem_bytes(sizeof(K), true, kPartIPTB, true, kPartNWB);
     set_smem_once(kern, sm);
@@ -1725,23 +1803,8 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   ba.order = any_order ? &hdr->order_mode : nullptr;
   {
     HG_TRACE("k_binbuild", st);
-    auto launch = [&](const BinCfg& c, uint32_t emin, const uint32_t* gate) {
-      BinArgs<K> x = ba;
-      x.emax = c.emax;
-      x.list = c.list;
-      x.has_pos = c.pos;
-      x.emin = emin;
-      x.gate = gate;
-      auto go = [&](auto kern) {
-        set_smem_once(kern, c.smem);
-        kern<<<c.grid, c.nt, c.smem, st>>>(x, map);
-      };
-      if (c.nt == 256) go(k_binbuild<K, Map, 256>);
-      else if (c.nt == 512) go(k_binbuild<K, Map, 512>);
-      else go(k_binbuild<K, Map, 1024>);
-    };
-    launch(bc, 0, nullptr);
-    if (bc.nt != bw.nt) launch(bw, bc.emax, wide_count);
+    binbuild_launch<K, Map>(ba, map, bc, 0, nullptr, st);
+    if (bc.nt != bw.nt) binbuild_launch<K, Map>(ba, map, bw, bc.emax, wide_count, st);
   }
   {
     const size_t sm = big_smem_bytes(sizeof(K), 1u << p.s);
@@ -1823,6 +1886,36 @@ bool make_slab_plan(const hg_config* cfg, uint64_t n, SlabPlan* p) {
   p->o_i = o;   o = align_up(o + ((size_t)n + 16) * 4);
   p->o_sub = o; o = align_up(o + p->sub.total);
   p->total = o;
+  // the same table as one two-level build (build_wide): bins of the slabs'
+  // size, up to 256 in each of up to 512 super-bins
+  Plan& w = p->wide;
+  w = Plan{};
+  const uint64_t nbins = ((p->V - 1) >> s_fit) + 1;
+  if (nbins > (1ull << 17)) return true;
+  w.kb = p->kb;
+  w.n = n;
+  w.V = p->V;
+  w.s = (uint32_t)s_fit;
+  w.sshift = 8;
+  w.nbins = (uint32_t)nbins;
+  w.nsb = (uint32_t)(((nbins - 1) >> w.sshift) + 1);
+  w.G = p->G;
+  w.chunk = p->chunk;
+  w.emax = p->sub.emax;
+  w.tpb = cfg->threads_per_bin;
+  o = sizeof(WsHeader);
+  w.o_H = o;      o = align_up(o + (size_t)w.G * w.nsb * 4);
+  w.o_C = o;      o = align_up(o + (size_t)w.G * w.nsb * 4);
+  w.o_CT = o;     o = align_up(o + (size_t)w.nsb * 4);
+  w.o_T = o;      o = align_up(o + (size_t)w.nbins * 4);
+  w.o_BS = o;     o = align_up(o + ((size_t)w.nbins + 1) * 4);
+  p->o_wcur = o;  o = align_up(o + (size_t)w.nbins * 4);
+  p->o_wsbs = o;  o = align_up(o + ((size_t)w.nsb + 1) * 4);
+  w.o_ovf = o;    o = align_up(o + (size_t)w.nbins * 4 + 16);
+  w.o_bk = o;     o = align_up(o + ((size_t)n + 16) * w.kb);
+  w.o_bi = o;     o = align_up(o + ((size_t)n + 16) * 4);
+  w.total = o;
+  p->total = std::max(p->total, o);
   return true;
 }
 
@@ -1835,6 +1928,112 @@ __global__ void k_fill_u32(uint32_t* __restrict__ a, uint64_t n, uint32_t v) {
 // are carried over to the caller's.
 __global__ void k_carry_status(const uint32_t* __restrict__ from, uint32_t* to) {
   if (*from) set_status(to, *from);
+}
+
+// Tables of more bins than one shared-memory histogram holds, implicit ids:
+// one two-level build all the same, with up to 512 super-bins in pass A and
+// the bin totals counted from pass A's output (k_hist_late).  The host reads
+// whether every bin fits the shared-memory bin build (one stream
+// synchronisation); if not, nothing is built (*done = false) and the slabs
+// take over.  Spares the slabs' stable partition of the whole input: build of
+// 2^30 uint32 keys 18.6 ms, of the same keys through the slabs 36.6 (explicit ids).
+template <typename K, typename Map>
+static hg_status build_wide(const SlabPlan& sp, const K* keys, uint32_t* offsets, K* csr_k, uint32_t* csr_i,
+                            uint8_t* ws, cudaStream_t st, Map map, bool* done) {
+  *done = false;
+  const Plan& p = sp.wide;
+  WsHeader* hdr = (WsHeader*)ws;
+  uint32_t* H = (uint32_t*)(ws + p.o_H);
+  uint32_t* C = (uint32_t*)(ws + p.o_C);
+  uint32_t* CT = (uint32_t*)(ws + p.o_CT);
+  uint32_t* T = (uint32_t*)(ws + p.o_T);
+  uint32_t* BS = (uint32_t*)(ws + p.o_BS);
+  uint32_t* cur = (uint32_t*)(ws + sp.o_wcur);
+  uint32_t* sbs = (uint32_t*)(ws + sp.o_wsbs);
+  uint32_t* ovf = (uint32_t*)(ws + p.o_ovf);
+  K* bk = (K*)(ws + p.o_bk);
+  uint32_t* bi = (uint32_t*)(ws + p.o_bi);
+  const DevInfo& di = dev_info();
+  const uint32_t sb_log2 = p.s + p.sshift;  // buckets per super-bin
+  {
+    const size_t sm = hist_stage_offset(p.nsb) + Map::kStageBytes;
+    auto kern = k_hist<K, Map>;
+    set_smem_once(kern, sm);
+    HG_TRACE("k_hist", st);
+    kern<<<p.G, kHistThreads, sm, st>>>(keys, p.n, p.chunk, sb_log2, p.nsb, 0, p.nsb, H, C, map,
+                                        (uint32_t)Map::kStageBytes);
+    colscan_launch(C, p.G, p.nsb, CT, st);
+    k_scan_bins<<<1, 1024, 0, st>>>(CT, p.nsb, sbs, 0xffffffffu, ovf, &hdr->ovf_count, ovf + p.nsb, 0, (uint32_t)p.n,
+                                    HugeArgs{}, nullptr);
+  }
+  PartArgs<K> a{};
+  a.in_k = keys;
+  a.out_k = csr_k;
+  a.out_i = csr_i;
+  a.n = p.n;
+  a.chunk = p.chunk;
+  a.G = p.G;
+  a.s = sb_log2;  // pass A and the late histogram know super-bins by their starts alone
+  a.nbins = p.nsb;
+  a.nsb = p.nsb;
+  a.C = C;
+  a.CT = CT;
+  a.BS = sbs;
+  a.status = &hdr->status;
+  {
+    HG_TRACE("k_partition_A", st);
+    partition_any<K, Map, false, false, PartA<K>, 512>(a, map, p.G, st);
+  }
+  a.in_k = csr_k;
+  a.in_i = csr_i;
+  a.out_k = bk;
+  a.out_i = bi;
+  a.s = p.s;
+  a.sshift = p.sshift;
+  a.nbins = p.nbins;
+  if (cudaMemsetAsync(T, 0, (size_t)p.nbins * 4, st) != cudaSuccess) return HG_ERR_CUDA;
+  {
+    HG_TRACE("k_hist_late", st);
+    const uint64_t pieces = (p.n + kLatePiece - 1) / kLatePiece;
+    k_hist_late<K, Map><<<(unsigned)std::min<uint64_t>(pieces, 4ull * di.sms), 512, 0, st>>>(a, T, map);
+  }
+  BinCfg bc, bw;
+  bin_configs<K>(p, true, &bc, &bw);
+  uint32_t* const wide_count = (uint32_t*)&hdr->counters[7];
+  {
+    HG_TRACE("k_scan_bins", st);
+    k_scan_bins<<<1, 1024, 0, st>>>(T, p.nbins, BS, bw.emax, ovf, &hdr->ovf_count, offsets, p.V, (uint32_t)p.n,
+                                    HugeArgs{}, &hdr->order_mode, bc.emax, bc.nt != bw.nt ? wide_count : nullptr, cur);
+  }
+  if (cudaPeekAtLastError() != cudaSuccess) return last_launch_status();
+  uint32_t order = 1;
+  if (cudaMemcpyAsync(&order, &hdr->order_mode, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) return HG_ERR_CUDA;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return HG_ERR_CUDA;
+  if (order != 0) return HG_OK;
+  *done = true;
+  a.BS = BS;
+  a.cur_bin = cur;
+  {
+    HG_TRACE("k_partition_B", st);
+    partition_b_any<K, Map>(a, map, st);
+  }
+  if (cudaPeekAtLastError() != cudaSuccess) return last_launch_status();
+  BinArgs<K> ba{};
+  ba.in_k = bk;
+  ba.in_i = bi;
+  ba.csr_k = csr_k;
+  ba.csr_i = csr_i;
+  ba.offsets = offsets;
+  ba.T = T;
+  ba.BS = BS;
+  ba.V = p.V;
+  ba.nbins = p.nbins;
+  ba.s = p.s;
+  ba.order = &hdr->order_mode;
+  HG_TRACE("k_binbuild", st);
+  binbuild_launch<K, Map>(ba, map, bc, 0, nullptr, st);
+  if (bc.nt != bw.nt) binbuild_launch<K, Map>(ba, map, bw, bc.emax, wide_count, st);
+  return last_launch_status();
 }
 
 template <typename K, typename Map>
@@ -1851,6 +2050,12 @@ hg_status build_slabs(const hg_config* cfg, const SlabPlan& p, const K* keys, co
   uint32_t* li = (uint32_t*)(ws + p.o_i);
   uint8_t* sub = ws + p.o_sub;
   const DevInfo& di = dev_info();
+  if (p.wide.total != 0 && ids == nullptr) {
+    bool done;
+    const hg_status rc = build_wide<K, Map>(p, keys, offsets, csr_k, csr_i, ws, st, map, &done);
+    if (rc != HG_OK || done) return rc;
+    if (cudaMemsetAsync(ws, 0, sizeof(WsHeader), st) != cudaSuccess) return HG_ERR_CUDA;
+  }
   // 1. slab of every key (bucket >> Ls), counted per input chunk
   {
     const size_t sm = hist_stage_offset(p.S) + Map::kStageBytes;
@@ -2182,19 +2387,16 @@ static uint32_t query_tile(int kb) {
                  : (uint32_t)(PartQ<uint32_t>::NT * PartQ<uint32_t>::IPT);
 }
 
-#ifndef HG_PROBE_GROUP_BITS
-#define HG_PROBE_GROUP_BITS 7  // log2 of the query groups (at most 8; 7 measured best at 2^28)
-#endif
 bool make_probe_plan(const hg_config* cfg, uint64_t table_n, uint64_t q, ProbePlan* p) {
   const DevInfo& di = dev_info();
   const int kb = cfg->key_type == HG_KEY_U64 ? 8 : 4;
   const uint64_t V = cfg->num_buckets;
-  // 256 groups (fewer only for V < 256): a group's slice of the table stays
-  // well below L2 up to 4 GB tables (a 2^28-key table gives 8 MB slices), and
-  // with many groups every output tile of the merge draws on many of them,
-  // which keeps its warps evenly loaded.
+  // 128 groups (fewer only for V < 128): a group's slice of the table stays
+  // well below L2 up to 2^28 buckets (16 MB slices at load 1), and with many
+  // groups every output tile of the merge draws on many of them, which keeps
+  // its warps evenly loaded.  256 groups above (32 MB slices at 2^30 buckets).
   (void)table_n;
-  int sg = ceil_log2_u64(V) - HG_PROBE_GROUP_BITS;
+  int sg = ceil_log2_u64(V) - (V <= (1ull << 28) ? 7 : 8);
   if (sg < 0) sg = 0;
   p->sg = (uint32_t)sg;
   p->ng = (uint32_t)(((V - 1) >> sg) + 1);
@@ -2277,9 +2479,19 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
   // the probe and the merge index by the grouped positions: none may run on
   // a query partition that was not launched
   if (cudaPeekAtLastError() != cudaSuccess) return last_launch_status();
-  hg_status rc = probe_launch<K, Map>(qk, q, t->d_offsets, (const K*)t->d_keys, qc, V, st, map,
-                                      Map::kNeedsPos ? qi : nullptr);
-  if (rc != HG_OK) return rc;
+  // The CTAs of a launch drift apart as they sweep the groups, and with them
+  // the table slices in use; where a few of these do not fit L2 together, a
+  // launch takes only so many queries (k_probe in all, one launch / launches
+  // of 2^26: uint32 keys 2^28 2.07 / 2.11 ms (slices of 16 MB), 2^30 30.5 /
+  // 8.9 (32 MB); uint64 2^28 2.70 / 2.28 (24 MB); 2500 batched tables 3.29 /
+  // 2.79 with launches of 2^25, 3.03 with 2^26).
+  const uint64_t slice = (4 * V + t->n * sizeof(K)) / p.ng;
+  const uint64_t step = Map::kNeedsPos ? 1ull << 25 : slice > (17ull << 20) ? 1ull << 26 : q;
+  for (uint64_t i = 0; i < q; i += step) {
+    hg_status rc = probe_launch<K, Map>(qk + i, std::min(q - i, step), t->d_offsets, (const K*)t->d_keys, qc + i, V,
+                                        st, map, Map::kNeedsPos ? qi + i : nullptr);
+    if (rc != HG_OK) return rc;
+  }
   {
     // every CTA merges a span of at least one block of outputs (in tiles of up to
     // kUnpermuteTile), so small batches still spread over the SMs
@@ -2313,7 +2525,7 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
 
 bool make_slab_probe_plan(const hg_config* cfg, uint64_t table_n, uint64_t q, SlabProbePlan* p) {
   const uint64_t V = cfg->num_buckets;
-  if (V <= (1ull << kSlabProbeLog2) || q == 0) return false;
+  if (V <= (1ull << kBinnedProbeLog2) || q == 0) return false;
   const DevInfo& di = dev_info();
   const int kb = cfg->key_type == HG_KEY_U64 ? 8 : 4;
   p->V = V;
@@ -2390,7 +2602,7 @@ hg_status probe_slabs(const hg_config* cfg, const SlabProbePlan& p, const hg_tab
     pa.CT = CT;
     pa.BS = GS;
     pa.status = &hdr->status;
-    pa.tile_counts = Map::kSkewed ? (uint16_t*)(ws + p.o_tc) : nullptr;
+    pa.tile_counts = (uint16_t*)(ws + p.o_tc);
     HG_TRACE("k_partition_Q", st);
     partition_any<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
   }
@@ -2422,15 +2634,9 @@ hg_status probe_slabs(const hg_config* cfg, const SlabProbePlan& p, const hg_tab
     const uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(blocks, (uint64_t)2 * di.sms));
     const uint64_t span = (blocks + grid - 1) / grid * kQueryBlock;
     HG_TRACE("k_unpermute", st);
-    if (Map::kSkewed) {
-      set_smem_once(k_unpermute_bal, (size_t)kUnpermuteTile * 4);
-      k_unpermute_bal<<<(unsigned)grid, kUnpermuteThreads, (size_t)kUnpermuteTile * 4, st>>>(
-          qi, qc, GS, p.S, (const uint16_t*)(ws + p.o_tc), p.ptile, q, span, counts);
-    } else {
-      auto kern = k_unpermute<1, 8>;
-      set_smem_once(kern, (size_t)kUnpermuteTile * 4);
-      kern<<<(unsigned)grid, kUnpermuteThreads, (size_t)kUnpermuteTile * 4, st>>>(qi, qc, GS, p.S, q, span, counts);
-    }
+    set_smem_once(k_unpermute_bal, (size_t)kUnpermuteTile * 4);  // a few slabs: a warp per group would idle most warps
+    k_unpermute_bal<<<(unsigned)grid, kUnpermuteThreads, (size_t)kUnpermuteTile * 4, st>>>(
+        qi, qc, GS, p.S, (const uint16_t*)(ws + p.o_tc), p.ptile, q, span, counts);
   }
   return last_launch_status();
 }

@@ -39,7 +39,7 @@ struct PartQ {  // queries: tiles of 8192 / 4096 (they divide kQueryBlock); two 
 };
 constexpr uint32_t kPartPiece = 8;  // pass B: most tiles a CTA takes at a time (1: 1.19 ms, 4: 1.11, 8: 1.08)
 constexpr uint32_t kMaxItemsPerCta = 128;  // pass B work items one CTA may own
-constexpr uint32_t kMaxBinsPerCta = 256;   // bins one bin-build CTA may own
+constexpr uint32_t kMaxBinsPerCta = 512;   // bins one bin-build CTA may own
 constexpr int kPartTile = 4096;  // smallest chunk of keys
 constexpr int kBinNW = 32;             // warps of the oversized-bin kernels (1024 threads)
 constexpr int kBigTile = 2048;         // tile of the oversized-bin kernel
@@ -82,7 +82,8 @@ struct SlabPlan {
   uint32_t Ls, S, G;
   uint64_t chunk;
   Plan sub;  // plan of a slab holding all n keys: the bound of every slab build's workspace
-  size_t o_H, o_C, o_CT, o_T, o_BS, o_ovf, o_k, o_i, o_sub, total;
+  Plan wide;  // the table as one two-level build (total 0: too many bins)
+  size_t o_H, o_C, o_CT, o_T, o_BS, o_ovf, o_k, o_i, o_sub, o_wcur, o_wsbs, total;
 };
 bool make_slab_plan(const hg_config* cfg, uint64_t n, SlabPlan* p);
 template <typename K, typename Map>
@@ -99,13 +100,14 @@ struct ProbePlan {
   size_t o_H, o_C, o_CT, o_GS, o_ovf, o_qk, o_qi, o_qc, o_tc, total;
 };
 bool make_probe_plan(const hg_config* cfg, uint64_t table_n, uint64_t q, ProbePlan* p);
-// Binned probe of a table of more than 2^kSlabProbeLog2 buckets: 128 query
+// Binned probe of a table of more than 2^kBinnedProbeLog2 buckets: 256 query
 // groups would leave each group a table slice too large for L2, so the
-// queries are first grouped by slab of 2^kSlabProbeLog2 buckets (the slabs a
-// large build relabels by), each slab's queries take the binned probe
-// against the slab's part of the table, and the counts are merged back to
-// query order.  The slab query counts are read back to the host between the
-// two steps (one stream synchronisation).
+// queries are first grouped by slab of 2^kSlabProbeLog2 buckets, each slab's
+// queries take the binned probe against the slab's part of the table, and
+// the counts are merged back to query order.  The slab query counts are read
+// back to the host between the two steps (one stream synchronisation).
+// (2^30 queries of 2^31 buckets, slabs of 2^28 / 2^30: 22.9 / 24.7 ms.)
+constexpr uint32_t kBinnedProbeLog2 = 30;
 constexpr uint32_t kSlabProbeLog2 = 28;
 struct SlabProbePlan {
   uint64_t V, q;
