@@ -127,7 +127,8 @@ hg_status hg_build(const hg_config* cfg, const void* d_keys, const uint32_t* d_i
   if (rc != HG_OK) return rc;
   if (ws_bytes < build_ws_bytes_of(cfg, n, kind, p, sp)) return HG_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
-  if (cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st) != cudaSuccess) return HG_ERR_CUDA;
+  // (the two-level build clears the header itself)
+  if ((n == 0 || kind != kBuildV2) && cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st) != cudaSuccess) return HG_ERR_CUDA;
   if (n == 0) {
     if (cudaMemsetAsync(d_offsets, 0, (size_t)(cfg->num_buckets + 1) * 4, st) != cudaSuccess) return HG_ERR_CUDA;
     return HG_OK;

@@ -11,7 +11,7 @@
 //                (Phase 2, "Bin Placement and Data Reorganization")
 //   k_binbuild   per bin, in shared memory: local bucket index, counting
 //                sort, CSR offsets and edges (Phase 3, "HashGraph Creation")
-//   k_binbuild_big  bins larger than shared memory, streamed by one CTA each
+//                bins larger than shared memory are streamed by one CTA each
 // The table comes out in the canonical order (bucket, then input position)
 // without atomics deciding any position: either both partitions are stable
 // and the bin build ranks each bucket by bin position, or (implicit ids and
@@ -74,7 +74,12 @@ bool make_plan_v2(const hg_config* cfg, uint64_t n, Plan* p) {
     const double bpb = n ? target * (double)V / (double)n : (double)V;
     s = bpb <= 1.0 ? 0 : (int)std::floor(std::log2(bpb));
   }
-  if (!cfg->bin_shift) s = std::min(s, (int)kMaxBinShift);
+  if (!cfg->bin_shift) {
+    s = std::min(s, (int)kMaxBinShift);
+    // small builds: 128 bins all the same, about one per SM, rather than a
+    // few large ones
+    s = std::min(s, std::max(0, ceil_log2_u64(V) - 7));
+  }
   s = std::max(s, ceil_log2_u64(V) - (int)kMaxBinsLog2);
   s = std::max(s, 0);
   if (s > (int)kMaxBinShift) return false;
@@ -131,14 +136,18 @@ __host__ __device__ inline size_t hist_stage_offset(uint32_t nbins) {
 }
 
 // Phase 1: per-chunk bin histogram in shared memory; per super-bin sums.
+// header (may be null): the workspace header, cleared here for the kernels
+// that follow.
 template <typename K, typename Map>
 __global__ void __launch_bounds__(kHistThreads) k_hist(const K* __restrict__ keys, uint64_t n,
                                                        uint64_t chunk, uint32_t s, uint32_t nbins,
                                                        uint32_t sshift, uint32_t nsb,
                                                        uint32_t* __restrict__ H,
                                                        uint32_t* __restrict__ C, Map map,
-                                                       uint32_t stage_bytes) {
+                                                       uint32_t stage_bytes, WsHeader* header) {
   extern __shared__ __align__(16) uint32_t hist[];
+  if (header != nullptr && blockIdx.x == 0 && threadIdx.x < sizeof(WsHeader) / 4)
+    reinterpret_cast<uint32_t*>(header)[threadIdx.x] = 0;
   map.init();
   map.stage((uint8_t*)hist + hist_stage_offset(nbins), stage_bytes);
   for (uint32_t i = threadIdx.x; i < nbins; i += blockDim.x) hist[i] = 0;
@@ -320,6 +329,59 @@ __global__ void __launch_bounds__(1024) k_scan_bins(const uint32_t* __restrict__
   }
 }
 
+// k_colscan and k_scan_bins in one, for builds of one partition pass (at most
+// 256 bins) and few chunks: thread = (bin, quarter of the chunks), every
+// count read once.  2^16 keys: one launch of 4 us for three of 10 us.
+constexpr uint32_t kScanSmallChunks = 64;
+__global__ void __launch_bounds__(1024) k_scan_small(uint32_t* __restrict__ C, uint32_t G, uint32_t nbins,
+                                                     uint32_t* __restrict__ CT, uint32_t* __restrict__ BS,
+                                                     uint32_t emax, uint32_t* __restrict__ ovf_list,
+                                                     uint32_t* __restrict__ ovf_count, uint32_t* __restrict__ offsets,
+                                                     uint64_t V, uint32_t n_end, uint32_t* order, uint32_t wide_lo,
+                                                     uint32_t* wide_count) {
+  constexpr uint32_t R = kScanSmallChunks / 4;
+  __shared__ uint32_t part[4][256];
+  __shared__ uint32_t wsum[32];
+  const uint32_t b = threadIdx.x & 255u, q = threadIdx.x >> 8;
+  uint32_t c[R], sum = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < R; ++i) {
+    const uint32_t g = q * R + i;
+    c[i] = b < nbins && g < G ? C[(uint64_t)g * nbins + b] : 0u;
+  }
+#pragma unroll
+  for (uint32_t i = 0; i < R; ++i) sum += c[i];
+  part[q][b] = sum;
+  __syncthreads();
+  uint32_t run = 0, t = 0;
+#pragma unroll
+  for (uint32_t i = 0; i < 4; ++i) {
+    run += i < q ? part[i][b] : 0u;
+    t += part[i][b];
+  }
+#pragma unroll
+  for (uint32_t i = 0; i < R; ++i) {
+    const uint32_t g = q * R + i;
+    if (b < nbins && g < G) C[(uint64_t)g * nbins + b] = run;
+    run += c[i];
+  }
+  uint32_t total;
+  const uint32_t start = block_excl_scan<uint32_t>(q == 0 ? t : 0u, wsum, &total);  // the first 256 threads' totals
+  if (q == 0 && b < nbins) {
+    CT[b] = t;
+    BS[b] = start;
+    if (wide_count && t > wide_lo && t <= emax) atomicAdd(wide_count, 1u);
+    if (t > emax) {
+      if (order) *order = 1u;
+      ovf_list[atomicAdd(ovf_count, 1u)] = b;
+    }
+  }
+  if (threadIdx.x == 0) {
+    BS[nbins] = total;
+    offsets[V] = n_end;
+  }
+}
+
 // Phase 2 (both passes).  Pass A: items are input chunks; digit = super-bin.
 // Pass B: items are (super-bin, group of gg consecutive chunks) sub-ranges of
 // pass A's output, contiguous in memory; digit = bin inside the super-bin.
@@ -353,14 +415,11 @@ struct PartArgs {
   uint16_t* tile_counts;
 };
 
-// The stable partition.  With a.order set, the build launches it and
-// k_partition_any, and the one that does not match the order mode written by
-// k_scan_bins returns at once: the unordered one runs only when every bin
-// fits the shared-memory bin build, which then restores the canonical order
-// by id.
-template <typename K, typename Map, bool PASS_B, int IPT, int NW, int MINB>
-__global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map map) {
-  if (a.order != nullptr && *(volatile const uint32_t*)a.order == 0u) return;
+// The stable partition.  The unordered one (partition_any) runs only when
+// every bin fits the shared-memory bin build, which then restores the
+// canonical order by id; k_scan_bins writes which it is (order mode).
+template <typename K, typename Map, bool PASS_B, int IPT, int NW>
+__device__ __forceinline__ void partition_stable(const PartArgs<K>& a, Map& map) {
   constexpr uint32_t TILE = NW * 32 * IPT;
   constexpr uint32_t TB = TILE + 16;
   static_assert(TILE <= 65536, "tile indexes are packed into 16 bits");
@@ -519,6 +578,15 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map 
   }
 }
 
+// The stable partition as a kernel of its own (explicit ids, pass B, slabs,
+// the sample sort): returns at once when the order mode (if there is one)
+// asks for the other.
+template <typename K, typename Map, bool PASS_B, int IPT, int NW, int MINB>
+__global__ void __launch_bounds__(NW * 32, MINB) k_partition(PartArgs<K> a, Map map) {
+  if (a.order != nullptr && *(volatile const uint32_t*)a.order == 0u) return;
+  partition_stable<K, Map, PASS_B, IPT, NW>(a, map);
+}
+
 // Shared memory of k_partition_any (see there).
 static size_t part_any_smem(int kb, bool ids, int tile, int digits) {
   return align_up((size_t)tile * (kb + 4 + (ids ? 1 : 0)), 16) + 4 * (size_t)digits * 4;
@@ -550,9 +618,8 @@ static size_t part_any_smem(int kb, bool ids, int tile, int digits) {
 // 2^28 uint32 keys, against tiles staged by TMA through a double buffer:
 // pass A 1.18 -> 0.96 ms, pass B 1.41 -> 1.08, queries 1.10 -> 0.92; 2^26
 // uint64 keys under the learned map 0.63 -> 0.47, 0.78 -> 0.46, 0.49 -> 0.41.
-template <typename K, typename Map, bool PASS_B, bool IDS, int DIG, int NT, int IPT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map map) {
-  if (a.order != nullptr && *(volatile const uint32_t*)a.order != 0u) return;
+template <typename K, typename Map, bool PASS_B, bool IDS, int DIG, int NT, int IPT>
+__device__ __forceinline__ void partition_any(const PartArgs<K>& a, Map& map) {
   constexpr uint32_t TILE = NT * IPT;
   static_assert(TILE <= 65536 && TILE % 16 == 0, "tile indexes are packed into 16 bits");
   static_assert(DIG == 256 || (DIG == 512 && !IDS && NT >= 512), "digits fit their packings");
@@ -735,6 +802,27 @@ __global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map m
   }
 }
 
+// ... as a kernel of its own; returns at once when the order mode (if there is
+// one) asks for the stable partition.
+template <typename K, typename Map, bool PASS_B, bool IDS, int DIG, int NT, int IPT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_partition_any(PartArgs<K> a, Map map) {
+  if (a.order != nullptr && *(volatile const uint32_t*)a.order != 0u) return;
+  partition_any<K, Map, PASS_B, IDS, DIG, NT, IPT>(a, map);
+}
+
+// Pass A of small builds with implicit ids: whichever the order mode asks
+// for, in one launch (a second one that returns at once costs 3 us).  Large
+// builds launch the two forms apart: together their code is slower (2^28
+// uint32 keys 1.01 against 0.96 ms).
+template <typename K, typename Map>
+__global__ void __launch_bounds__(PartA<K>::NT, PartA<K>::MINB) k_partition_a(PartArgs<K> a, Map map) {
+  static_assert(PartA<K>::NT == kPartNW * 32, "both forms have the same threads");
+  if (*(volatile const uint32_t*)a.order == 0u)
+    partition_any<K, Map, false, false, 256, PartA<K>::NT, PartA<K>::IPT>(a, map);
+  else
+    partition_stable<K, Map, false, part_ipt_keys<K>(), kPartNW>(a, map);
+}
+
 // Bin totals after pass A, for builds of more bins than one shared-memory
 // histogram of the whole input holds: the CTAs take equal pieces of pass A's
 // output in turn and count a piece's bins super-bin by super-bin (up to 256
@@ -795,7 +883,114 @@ struct BinArgs {
   bool has_pos;           // room for bin positions: the launch can rank by position
   const uint32_t* order;  // order mode word (null: partitions were stable); see k_partition
   const uint32_t* gate;   // null, or a count written by k_scan_bins: no bin for the launch when it is 0
+  const uint32_t* ovf_list;   // launch of 1024-thread CTAs: bins for build_big_bins, and their number
+  const uint32_t* ovf_count;  // (null: none)
 };
+
+// Streams edges [start, start + len) of a bin in tiles of kBigTile, sorts
+// every tile stably by local bucket and appends each run at its bucket's
+// cursor (cur: absolute CSR positions of the bin's nb buckets, advanced).
+// Tiles follow input order and each is sorted stably, so every bucket keeps
+// ascending input position.
+template <typename K, typename Map, int NW>
+__device__ __forceinline__ void stream_runs(const BinArgs<K>& a, const Map& map, uint32_t start, uint32_t len,
+                                            uint64_t bucket0, uint32_t nb, uint32_t* cur, uint8_t* sp) {
+  constexpr int IPT = kBigTile / (NW * 32);
+  K* tk = (K*)sp; sp += (size_t)kBigTile * sizeof(K);
+  uint32_t* ti = (uint32_t*)sp; sp += (size_t)kBigTile * 4;
+  uint16_t* lb = (uint16_t*)sp; sp += kBigTile * 2;
+  uint16_t* tmp = (uint16_t*)sp; sp += kBigTile * 2;
+  uint16_t* perm = (uint16_t*)sp; sp += kBigTile * 2;
+  uint16_t* slb = (uint16_t*)sp; sp += kBigTile * 2;
+  sp = (uint8_t*)(((uintptr_t)sp + 15) & ~(uintptr_t)15);
+  uint32_t* wc = (uint32_t*)sp; sp += rank_words<NW>() * 4;
+  uint32_t* wsum = (uint32_t*)sp;
+  for (uint32_t t0 = 0; t0 < len; t0 += kBigTile) {
+    const uint32_t cnt = min((uint32_t)kBigTile, len - t0);
+    for (uint32_t e = threadIdx.x; e < cnt; e += blockDim.x) {
+      const K key = a.in_k[start + t0 + e];
+      const uint32_t id = a.in_i[start + t0 + e];
+      tk[e] = key;
+      ti[e] = id;
+      lb[e] = (uint16_t)(map(key, id) - (uint32_t)bucket0);
+    }
+    __syncthreads();
+    const uint16_t* sorted = sort_positions_by_bucket<IPT, NW>(lb, cnt, nb, tmp, perm, wc, wsum);
+    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) slb[j] = lb[sorted[j]];
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
+      const uint16_t l = slb[j];
+      uint32_t lo = 0, hi = j;  // first index with slb == l
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (slb[mid] < l) lo = mid + 1; else hi = mid;
+      }
+      const uint32_t g = cur[l] + (j - lo);
+      const uint32_t p = sorted[j];
+      a.csr_k[g] = tk[p];
+      a.csr_i[g] = map.out_id(ti[p]);
+    }
+    __syncthreads();
+    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
+      const uint16_t l = slb[j];
+      if (j + 1 == cnt || slb[j + 1] != l) {
+        uint32_t lo = 0, hi = j;
+        while (lo < hi) {
+          const uint32_t mid = (lo + hi) >> 1;
+          if (slb[mid] < l) lo = mid + 1; else hi = mid;
+        }
+        cur[l] += j - lo + 1;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Local-bucket counts of edges [start, start + len) of a bin into cur[]
+// (zeroed first).  Equal buckets of a warp are merged by __match_any_sync,
+// so a bucket holding most of the bin (duplicates) costs one shared-memory
+// atomic per warp instead of one per edge.
+template <typename K, typename Map>
+__device__ __forceinline__ void count_local(const BinArgs<K>& a, const Map& map, uint32_t start, uint32_t len,
+                                            uint64_t bucket0, uint32_t nb, uint32_t* cur) {
+  for (uint32_t v = threadIdx.x; v < nb; v += blockDim.x) cur[v] = 0;
+  __syncthreads();
+  const uint32_t lane = lane_id();
+  for (uint32_t base = threadIdx.x & ~31u; base < len; base += blockDim.x) {
+    const uint32_t e = base + lane;
+    const bool valid = e < len;
+    const uint32_t l = valid ? map(a.in_k[start + e], a.in_i[start + e]) - (uint32_t)bucket0 : 0xffffffffu;
+    const uint32_t peers = __match_any_sync(kFull, l);
+    if (valid && lane == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&cur[l], (uint32_t)__popc(peers));
+  }
+  __syncthreads();
+}
+
+// Bins too large for shared memory (duplicates, skew, tiny V) with at most
+// kHugeSeg edges: one CTA per bin counts its local buckets, writes the bin's
+// offsets and streams the bin (stream_runs).  Called by the bin build's launch
+// of 1024-thread CTAs after its own bins.
+template <typename K, typename Map>
+__device__ __noinline__ void build_big_bins(BinArgs<K> a, uint32_t novf, Map map, uint8_t* smem) {
+  const uint32_t nbmax = 1u << a.s;
+  uint32_t* cur = (uint32_t*)smem;
+  uint8_t* rest = smem + align_up((size_t)nbmax * 4, 16);
+  uint32_t* wsum = (uint32_t*)(rest + big_rest_bytes(sizeof(K)) - 32 * 4);
+  for (uint32_t k = blockIdx.x; k < novf; k += gridDim.x) {
+    const uint32_t b = a.ovf_list[k];
+    const uint32_t E = a.T[b], start = a.BS[b];
+    const uint64_t bucket0 = (uint64_t)b << a.s;
+    const uint32_t nb = (uint32_t)min((uint64_t)nbmax, a.V - bucket0);
+    count_local(a, map, start, E, bucket0, nb, cur);
+    block_excl_scan_smem(cur, (int)nb, wsum);
+    for (uint32_t v = threadIdx.x; v < nb; v += blockDim.x) {
+      a.offsets[bucket0 + v] = a.pos_base + start + cur[v];
+      cur[v] += start;
+    }
+    __syncthreads();
+    stream_runs<K, Map, kBinNW>(a, map, start, E, bucket0, nb, cur, rest);
+  }
+}
 
 // Edges per thread of the bin build: a CTA of NT threads builds bins of up to
 // NT * bin_ipt<K>() edges (9216 uint32 or 7168 uint64 edges with 512 threads).
@@ -891,10 +1086,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_binbuild(BinArgs<K> a, Map ma
   const bool pos = a.order == nullptr || *(volatile const uint32_t*)a.order != 0u;
   if (pos && !a.has_pos) return;
   uint32_t emin = a.emin;
+  bool idle = false;  // no bin for this launch
   if (emin != 0) {  // second launch
     if (pos && a.order != nullptr) emin = 0;  // the first launch took no bin
-    else if (*(volatile const uint32_t*)a.gate == 0u) return;
+    else idle = *(volatile const uint32_t*)a.gate == 0u;
   }
+  const uint32_t novf = NT == kBinNW * 32 && a.ovf_count != nullptr ? *(volatile const uint32_t*)a.ovf_count : 0u;
+  if (idle && novf == 0) return;
   extern __shared__ __align__(16) uint8_t smem[];
   uint8_t* sp = smem;
   K* const ks0 = (K*)sp; sp += (size_t)(a.emax + 4) * sizeof(K);
@@ -918,7 +1116,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_binbuild(BinArgs<K> a, Map ma
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   // Bins blockIdx.x, +gridDim.x, ...: starts and sizes gathered once, so the
   // loop below needs no global loads to find its next bin.
-  const uint32_t nmine = blockIdx.x < a.nbins ? (a.nbins - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
+  const uint32_t nmine =
+      !idle && blockIdx.x < a.nbins ? (a.nbins - blockIdx.x + gridDim.x - 1) / gridDim.x : 0u;
   for (uint32_t j = tid; j < nmine; j += NT) {
     const uint32_t bb = blockIdx.x + j * gridDim.x;
     bl_start[j] = a.BS[bb];
@@ -1219,6 +1418,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_binbuild(BinArgs<K> a, Map ma
     clear();
     __syncthreads();
   }
+  if (NT == kBinNW * 32 && novf != 0) {
+    __syncthreads();
+    build_big_bins<K, Map>(a, novf, map, smem);
+  }
 }
 
 // Bin-build launch configuration.
@@ -1277,114 +1480,6 @@ static void bin_configs(const Plan& p, bool by_id, BinCfg* first, BinCfg* second
   *first = bin_config<K>(p, by_id);
   *second = bin_config_for<K>(p, 1024, true);
   first->emax = std::min(first->emax, second->emax);
-}
-
-// Streams edges [start, start + len) of a bin in tiles of kBigTile, sorts
-// every tile stably by local bucket and appends each run at its bucket's
-// cursor (cur: absolute CSR positions of the bin's nb buckets, advanced).
-// Tiles follow input order and each is sorted stably, so every bucket keeps
-// ascending input position.
-template <typename K, typename Map, int NW>
-__device__ __forceinline__ void stream_runs(const BinArgs<K>& a, const Map& map, uint32_t start, uint32_t len,
-                                            uint64_t bucket0, uint32_t nb, uint32_t* cur, uint8_t* sp) {
-  constexpr int IPT = kBigTile / (NW * 32);
-  K* tk = (K*)sp; sp += (size_t)kBigTile * sizeof(K);
-  uint32_t* ti = (uint32_t*)sp; sp += (size_t)kBigTile * 4;
-  uint16_t* lb = (uint16_t*)sp; sp += kBigTile * 2;
-  uint16_t* tmp = (uint16_t*)sp; sp += kBigTile * 2;
-  uint16_t* perm = (uint16_t*)sp; sp += kBigTile * 2;
-  uint16_t* slb = (uint16_t*)sp; sp += kBigTile * 2;
-  sp = (uint8_t*)(((uintptr_t)sp + 15) & ~(uintptr_t)15);
-  uint32_t* wc = (uint32_t*)sp; sp += rank_words<NW>() * 4;
-  uint32_t* wsum = (uint32_t*)sp;
-  for (uint32_t t0 = 0; t0 < len; t0 += kBigTile) {
-    const uint32_t cnt = min((uint32_t)kBigTile, len - t0);
-    for (uint32_t e = threadIdx.x; e < cnt; e += blockDim.x) {
-      const K key = a.in_k[start + t0 + e];
-      const uint32_t id = a.in_i[start + t0 + e];
-      tk[e] = key;
-      ti[e] = id;
-      lb[e] = (uint16_t)(map(key, id) - (uint32_t)bucket0);
-    }
-    __syncthreads();
-    const uint16_t* sorted = sort_positions_by_bucket<IPT, NW>(lb, cnt, nb, tmp, perm, wc, wsum);
-    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) slb[j] = lb[sorted[j]];
-    __syncthreads();
-    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const uint16_t l = slb[j];
-      uint32_t lo = 0, hi = j;  // first index with slb == l
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (slb[mid] < l) lo = mid + 1; else hi = mid;
-      }
-      const uint32_t g = cur[l] + (j - lo);
-      const uint32_t p = sorted[j];
-      a.csr_k[g] = tk[p];
-      a.csr_i[g] = map.out_id(ti[p]);
-    }
-    __syncthreads();
-    for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const uint16_t l = slb[j];
-      if (j + 1 == cnt || slb[j + 1] != l) {
-        uint32_t lo = 0, hi = j;
-        while (lo < hi) {
-          const uint32_t mid = (lo + hi) >> 1;
-          if (slb[mid] < l) lo = mid + 1; else hi = mid;
-        }
-        cur[l] += j - lo + 1;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Local-bucket counts of edges [start, start + len) of a bin into cur[]
-// (zeroed first).  Equal buckets of a warp are merged by __match_any_sync,
-// so a bucket holding most of the bin (duplicates) costs one shared-memory
-// atomic per warp instead of one per edge.
-template <typename K, typename Map>
-__device__ __forceinline__ void count_local(const BinArgs<K>& a, const Map& map, uint32_t start, uint32_t len,
-                                            uint64_t bucket0, uint32_t nb, uint32_t* cur) {
-  for (uint32_t v = threadIdx.x; v < nb; v += blockDim.x) cur[v] = 0;
-  __syncthreads();
-  const uint32_t lane = lane_id();
-  for (uint32_t base = threadIdx.x & ~31u; base < len; base += blockDim.x) {
-    const uint32_t e = base + lane;
-    const bool valid = e < len;
-    const uint32_t l = valid ? map(a.in_k[start + e], a.in_i[start + e]) - (uint32_t)bucket0 : 0xffffffffu;
-    const uint32_t peers = __match_any_sync(kFull, l);
-    if (valid && lane == (uint32_t)(__ffs(peers) - 1)) atomicAdd(&cur[l], (uint32_t)__popc(peers));
-  }
-  __syncthreads();
-}
-
-// Bins too large for shared memory (duplicates, skew, tiny V) with at most
-// kHugeSeg edges: one CTA per bin counts its local buckets, writes the bin's
-// offsets and streams the bin (stream_runs).
-template <typename K, typename Map>
-__global__ void __launch_bounds__(kBinNW * 32, 1) k_binbuild_big(BinArgs<K> a, const uint32_t* ovf_list,
-                                                               const uint32_t* ovf_count, Map map) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  map.init();
-  const uint32_t nbmax = 1u << a.s;
-  uint32_t* cur = (uint32_t*)smem;
-  uint8_t* rest = smem + align_up((size_t)nbmax * 4, 16);
-  uint32_t* wsum = (uint32_t*)(rest + big_rest_bytes(sizeof(K)) - 32 * 4);
-  const uint32_t novf = *ovf_count;
-  for (uint32_t k = blockIdx.x; k < novf; k += gridDim.x) {
-    const uint32_t b = ovf_list[k];
-    const uint32_t E = a.T[b], start = a.BS[b];
-    const uint64_t bucket0 = (uint64_t)b << a.s;
-    const uint32_t nb = (uint32_t)min((uint64_t)nbmax, a.V - bucket0);
-    count_local(a, map, start, E, bucket0, nb, cur);
-    block_excl_scan_smem(cur, (int)nb, wsum);
-    for (uint32_t v = threadIdx.x; v < nb; v += blockDim.x) {
-      a.offsets[bucket0 + v] = a.pos_base + start + cur[v];
-      cur[v] += start;
-    }
-    __syncthreads();
-    stream_runs<K, Map, kBinNW>(a, map, start, E, bucket0, nb, cur, rest);
-  }
 }
 
 // Bins above kHugeSeg edges, split into segments of kHugeSeg edges (rows).
@@ -1620,7 +1715,7 @@ static void set_smem_once(F* kernel, size_t bytes) {
 // Launches k_partition_any with the tile of geometry T; the map's tables are
 // staged only where T::MINB CTAs still fit an SM.
 template <typename K, typename Map, bool PASS_B, bool IDS, typename T, int DIG = 256>
-static void partition_any(PartArgs<K> a, Map map, unsigned grid, cudaStream_t st) {
+static void partition_any_launch(PartArgs<K> a, Map map, unsigned grid, cudaStream_t st) {
   const DevInfo& di = dev_info();
   const size_t own = part_any_smem(sizeof(K), IDS, T::NT * T::IPT, DIG);
   a.stage_bytes = own + Map::kStageBytes + di.smem_reserved <= (size_t)di.smem_per_sm / T::MINB ? (uint32_t)Map::kStageBytes : 0u;
@@ -1637,7 +1732,7 @@ static void partition_b_any(PartArgs<K> a, Map map, cudaStream_t st) {
   const uint64_t resident = (uint64_t)PartB<K>::MINB * dev_info().sms, tiles = (a.n + tile - 1) / tile;
   a.piece = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(kPartPiece, tiles / (4 * resident)));
   const uint64_t pieces = (tiles + a.piece - 1) / a.piece;
-  partition_any<K, Map, true, true, PartB<K>>(a, map, (unsigned)std::min(pieces, resident), st);
+  partition_any_launch<K, Map, true, true, PartB<K>>(a, map, (unsigned)std::min(pieces, resident), st);
 }
 
 // One bin-build launch (k_binbuild): bins of more than emin edges (0: all) up
@@ -1668,7 +1763,6 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   uint32_t* H = (uint32_t*)(ws + p.o_H);
   uint32_t* C = (uint32_t*)(ws + p.o_C);
   uint32_t* CT = (uint32_t*)(ws + p.o_CT);
-  uint32_t* T = (uint32_t*)(ws + p.o_T);
   uint32_t* BS = (uint32_t*)(ws + p.o_BS);
   uint32_t* ovf = (uint32_t*)(ws + p.o_ovf);
   K* bk = (K*)(ws + p.o_bk);
@@ -1682,18 +1776,21 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     {
       HG_TRACE("k_hist", st);
       kern<<<p.G, kHistThreads, sm, st>>>(keys, p.n, p.chunk, p.s, p.nbins, p.sshift, p.nsb, H, C, map,
-                                          (uint32_t)Map::kStageBytes);
+                                          (uint32_t)Map::kStageBytes, hdr);
     }
   }
-  {
+  // With one pass a super-bin is a bin: C, CT serve for H, T.
+  const bool two = p.sshift > 0;
+  uint32_t* const T = two ? (uint32_t*)(ws + p.o_T) : CT;
+  const bool small = !two && p.G <= kScanSmallChunks && p.nbins <= 256;
+  if (two) {
     HG_TRACE("k_colscan", st);
     colscan_launch(H, p.G, p.nbins, T, st);
   }
-  {
+  if (!small) {
     HG_TRACE("k_colscan", st);
     colscan_launch(C, p.G, p.nsb, CT, st);
   }
-  const bool two = p.sshift > 0;
   // Implicit ids are input positions, so the bin build can restore the
   // canonical order (ascending position in every bucket) from the ids
   // alone; then, unless k_scan_bins finds a bin too large for the
@@ -1704,9 +1801,15 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   BinCfg bc, bw;
   bin_configs<K>(p, any_order, &bc, &bw);
   const uint32_t emax_all = bw.emax;
+  const bool may_overflow = p.n > emax_all;  // else no bin can be too large for shared memory
   // bins for the bin build's second launch, counted by k_scan_bins
   uint32_t* const wide_count = (uint32_t*)&hdr->counters[7];
-  {
+  if (small) {
+    HG_TRACE("k_scan_bins", st);
+    k_scan_small<<<1, 1024, 0, st>>>(C, p.G, p.nbins, CT, BS, emax_all, ovf, &hdr->ovf_count, offsets, p.V,
+                                     pos_base + (uint32_t)p.n, any_order ? &hdr->order_mode : nullptr, bc.emax,
+                                     bc.nt != bw.nt ? wide_count : nullptr);
+  } else {
     HG_TRACE("k_scan_bins", st);
     HugeArgs h{};
     // below kHugeMinN keys every oversized bin goes to the one-CTA path (at
@@ -1721,7 +1824,7 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     // launch included) go to the oversized-bin kernels
     k_scan_bins<<<1, 1024, 0, st>>>(T, p.nbins, BS, emax_all, ovf, &hdr->ovf_count, offsets, p.V,
                                     pos_base + (uint32_t)p.n, h, any_order ? &hdr->order_mode : nullptr, bc.emax,
-                                    bc.nt != bw.nt ? wide_count : nullptr, any_order ? H : nullptr);
+                                    bc.nt != bw.nt ? wide_count : nullptr, any_order && two ? H : nullptr);
   }
 
   PartArgs<K> pa{};
@@ -1748,18 +1851,26 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   {
     pa.order = any_order ? &hdr->order_mode : nullptr;
     HG_TRACE("k_partition_A", st);
-    if (any_order) {
-      if (ids == nullptr) partition_any<K, Map, false, false, PartA<K>>(pa, map, p.G, st);
-      else partition_any<K, Map, false, true, PartB<K>>(pa, map, p.G, st);
-    }
     // the map's tables are staged only where they fit next to the tile
     constexpr int ipt = part_ipt_keys<K>();
-    auto kern = k_partition<K, Map, false, ipt, kPartNW, part_minb_keys<K>()>;
     PartArgs<K> x = pa;
     const size_t own = part_smem_bytes(sizeof(K), ids != nullptr, ipt, false, kPartNW);
-    x.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
-    set_smem_once(kern, own + x.stage_bytes);
-    kern<<<p.G, kPartNW * 32, own + x.stage_bytes, st>>>(x, map);
+    if (ids == nullptr && p.n < kHugeMinN) {
+      const size_t need = std::max(own, part_any_smem(sizeof(K), false, PartA<K>::NT * PartA<K>::IPT, 256));
+      const size_t cap = std::min((size_t)di.max_smem_optin,
+                                  (size_t)di.smem_per_sm / PartA<K>::MINB - (size_t)di.smem_reserved);
+      x.stage_bytes = need + Map::kStageBytes <= cap ? (uint32_t)Map::kStageBytes : 0u;
+      auto kern = k_partition_a<K, Map>;
+      set_smem_once(kern, need + x.stage_bytes);
+      kern<<<p.G, kPartNW * 32, need + x.stage_bytes, st>>>(x, map);
+    } else {
+      if (ids == nullptr) partition_any_launch<K, Map, false, false, PartA<K>>(pa, map, p.G, st);
+      else if (any_order) partition_any_launch<K, Map, false, true, PartB<K>>(pa, map, p.G, st);
+      auto kern = k_partition<K, Map, false, ipt, kPartNW, part_minb_keys<K>()>;
+      x.stage_bytes = own + Map::kStageBytes <= (size_t)di.max_smem_optin ? (uint32_t)Map::kStageBytes : 0u;
+      set_smem_once(kern, own + x.stage_bytes);
+      kern<<<p.G, kPartNW * 32, own + x.stage_bytes, st>>>(x, map);
+    }
   }
   if (two) {
     PartArgs<K> pb = pa;
@@ -1775,14 +1886,16 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
     const uint64_t items = (uint64_t)p.nsb * pb.ngroups;
     HG_TRACE("k_partition_B", st);
     if (any_order) partition_b_any<K, Map>(pb, map, st);
-    auto kern = k_partition<K, Map, true, kPartIPTB, kPartNWB, kPartMinBlocksB>;
-    const size_t sm = part_smem_bytes(sizeof(K), true, kPartIPTB, true, kPartNWB);
-    set_smem_once(kern, sm);
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPartNWB * 32, sm);
-    unsigned grid = (unsigned)std::min<uint64_t>(items, (uint64_t)std::max(1, per_sm) * di.sms);
-    grid = (unsigned)std::max<uint64_t>(grid, (items + kMaxItemsPerCta - 1) / kMaxItemsPerCta);
-    kern<<<grid, kPartNWB * 32, sm, st>>>(pb, map);
+    if (!any_order || may_overflow) {
+      auto kern = k_partition<K, Map, true, kPartIPTB, kPartNWB, kPartMinBlocksB>;
+      const size_t sm = part_smem_bytes(sizeof(K), true, kPartIPTB, true, kPartNWB);
+      set_smem_once(kern, sm);
+      int per_sm = 0;
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPartNWB * 32, sm);
+      unsigned grid = (unsigned)std::min<uint64_t>(items, (uint64_t)std::max(1, per_sm) * di.sms);
+      grid = (unsigned)std::max<uint64_t>(grid, (items + kMaxItemsPerCta - 1) / kMaxItemsPerCta);
+      kern<<<grid, kPartNWB * 32, sm, st>>>(pb, map);
+    }
   }
   // A partition that could not be launched (say, a tile geometry built in at
   // compile time that needs more shared memory than a CTA may have) left the
@@ -1801,20 +1914,17 @@ hg_status build_v2(const Plan& p, const K* keys, const uint32_t* ids, uint32_t* 
   ba.s = p.s;
   ba.pos_base = pos_base;
   ba.order = any_order ? &hdr->order_mode : nullptr;
+  if (may_overflow) {  // (with room for them in the launch of 1024-thread CTAs)
+    ba.ovf_list = ovf;
+    ba.ovf_count = &hdr->ovf_count;
+    const size_t big = big_smem_bytes(sizeof(K), 1u << p.s);
+    bw.smem = std::max(bw.smem, big);
+    if (bc.nt == bw.nt) bc.smem = std::max(bc.smem, big);
+  }
   {
     HG_TRACE("k_binbuild", st);
     binbuild_launch<K, Map>(ba, map, bc, 0, nullptr, st);
     if (bc.nt != bw.nt) binbuild_launch<K, Map>(ba, map, bw, bc.emax, wide_count, st);
-  }
-  {
-    const size_t sm = big_smem_bytes(sizeof(K), 1u << p.s);
-    auto kern = k_binbuild_big<K, Map>;
-    set_smem_once(kern, sm);
-    const unsigned grid = (unsigned)std::min<uint64_t>(p.nbins, (uint64_t)di.sms);
-    {
-      HG_TRACE("k_binbuild_big", st);
-      kern<<<grid, kBinNW * 32, sm, st>>>(ba, ovf, &hdr->ovf_count, map);
-    }
   }
   if (p.n >= kHugeMinN) {
     // bins above kHugeSeg edges (duplicates): several CTAs per bin
@@ -1961,7 +2071,7 @@ static hg_status build_wide(const SlabPlan& sp, const K* keys, uint32_t* offsets
     set_smem_once(kern, sm);
     HG_TRACE("k_hist", st);
     kern<<<p.G, kHistThreads, sm, st>>>(keys, p.n, p.chunk, sb_log2, p.nsb, 0, p.nsb, H, C, map,
-                                        (uint32_t)Map::kStageBytes);
+                                        (uint32_t)Map::kStageBytes, nullptr);
     colscan_launch(C, p.G, p.nsb, CT, st);
     k_scan_bins<<<1, 1024, 0, st>>>(CT, p.nsb, sbs, 0xffffffffu, ovf, &hdr->ovf_count, ovf + p.nsb, 0, (uint32_t)p.n,
                                     HugeArgs{}, nullptr);
@@ -1982,7 +2092,7 @@ static hg_status build_wide(const SlabPlan& sp, const K* keys, uint32_t* offsets
   a.status = &hdr->status;
   {
     HG_TRACE("k_partition_A", st);
-    partition_any<K, Map, false, false, PartA<K>, 512>(a, map, p.G, st);
+    partition_any_launch<K, Map, false, false, PartA<K>, 512>(a, map, p.G, st);
   }
   a.in_k = csr_k;
   a.in_i = csr_i;
@@ -2063,7 +2173,7 @@ hg_status build_slabs(const hg_config* cfg, const SlabPlan& p, const K* keys, co
     set_smem_once(kern, sm);
     HG_TRACE("k_hist_slab", st);
     kern<<<p.G, kHistThreads, sm, st>>>(keys, p.n, p.chunk, p.Ls, p.S, 0, p.S, H, C, map,
-                                        (uint32_t)Map::kStageBytes);
+                                        (uint32_t)Map::kStageBytes, nullptr);
     colscan_launch(H, p.G, p.S, T, st);
     colscan_launch(C, p.G, p.S, CT, st);
     k_scan_bins<<<1, 1024, 0, st>>>(T, p.S, BS, 0xffffffffu, ovf, &hdr->ovf_count, ovf + p.S, 0, (uint32_t)p.n,
@@ -2442,7 +2552,7 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
     set_smem_once(kern, sm);
     HG_TRACE("k_hist_Q", st);
     kern<<<p.G, kHistThreads, sm, st>>>(queries, q, p.chunk, p.sg, p.ng, 0, p.ng, H, C, map,
-                                        (uint32_t)Map::kStageBytes);
+                                        (uint32_t)Map::kStageBytes, nullptr);
   }
   {
     HG_TRACE("k_colscan_Q", st);
@@ -2474,7 +2584,7 @@ hg_status probe_binned_impl(const ProbePlan& p, uint64_t V, const hg_table* t, c
   pa.tile_counts = Map::kSkewed ? (uint16_t*)(ws + p.o_tc) : nullptr;
   {
     HG_TRACE("k_partition_Q", st);
-    partition_any<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
+    partition_any_launch<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
   }
   // the probe and the merge index by the grouped positions: none may run on
   // a query partition that was not launched
@@ -2579,7 +2689,7 @@ hg_status probe_slabs(const hg_config* cfg, const SlabProbePlan& p, const hg_tab
     set_smem_once(kern, sm);
     HG_TRACE("k_hist_Q", st);
     kern<<<p.G, kHistThreads, sm, st>>>(queries, q, p.chunk, p.Ls, p.S, 0, p.S, H, C, map,
-                                        (uint32_t)Map::kStageBytes);
+                                        (uint32_t)Map::kStageBytes, nullptr);
     colscan_launch(C, p.G, p.S, CT, st);
     k_scan_bins<<<1, 1024, 0, st>>>(CT, p.S, GS, 0xffffffffu, ovf, &hdr->ovf_count, ovf + p.S, 0, (uint32_t)q,
                                     HugeArgs{}, nullptr);
@@ -2604,7 +2714,7 @@ hg_status probe_slabs(const hg_config* cfg, const SlabProbePlan& p, const hg_tab
     pa.status = &hdr->status;
     pa.tile_counts = (uint16_t*)(ws + p.o_tc);
     HG_TRACE("k_partition_Q", st);
-    partition_any<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
+    partition_any_launch<K, Map, false, false, PartQ<K>>(pa, map, p.G, st);
   }
   if (cudaPeekAtLastError() != cudaSuccess) return last_launch_status();  // partition not launched
   // 2. slab query counts to the host, then the binned probe of every slab
@@ -2711,7 +2821,7 @@ hg_status radix_sort_u64(uint64_t* keys, uint64_t n, uint8_t* ws, cudaStream_t s
     RadixByteMap map{8 * pass};
     {
       HG_TRACE("k_radix_hist", st);
-      kh<<<G, kHistThreads, hsm, st>>>(src, n, chunk, 0, 256, 0, 256, H, C, map, 0u);
+      kh<<<G, kHistThreads, hsm, st>>>(src, n, chunk, 0, 256, 0, 256, H, C, map, 0u, nullptr);
     }
     {
       HG_TRACE("k_radix_scan", st);
