@@ -296,8 +296,9 @@ hg_status hg_learned_judge(const hg_config* cfg, const void* d_keys, uint64_t n,
  *   HG_ERR_UNSUPPORTED).
  * hg_batch_run: enqueues the batch on `stream`.  Tables are grouped into
  *   waves whose buckets fit 2^15 bins of the bin size; per wave one
- *   two-level build (Alg. 2) and one binned probe over the wave's slice of
- *   the common bucket space.  The launch sequence is captured into a CUDA
+ *   two-level build (Alg. 2) and one probe over the wave's slice of the
+ *   common bucket space (binned where a table of the wave takes more than
+ *   64 MB).  The launch sequence is captured into a CUDA
  *   graph on the first call with a given set of buffers and configuration
  *   and replayed by later calls with the same ones.
  * hg_batch_run_eager: the same launch sequence enqueued directly, without

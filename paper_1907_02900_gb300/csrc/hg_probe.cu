@@ -131,7 +131,9 @@ using ReaderOf = TableReader<!Map::kSkewed && !Map::kNeedsPos>;
 // the table stays in L2 while it is needed: the table is read from DRAM
 // once.  (A grid of two waves sweeps every group twice and reads the table
 // twice.)  Each thread loads its next query one sweep ahead, so the query's
-// DRAM latency is not on its chain of dependent loads.
+// DRAM latency is not on its chain of dependent loads.  run (batched tables
+// only): consecutive blocks of queries a CTA takes at a time, which belong to
+// the same table mostly when the queries are in their own order.
 //
 // Bound by L1 tag look-ups and L2: one random access per lane takes a cycle
 // whatever its width (a warp's 32 take 34 cycles for 4 to 32 bytes, through
@@ -143,18 +145,27 @@ template <typename K, typename Map>
 __global__ void __launch_bounds__(kProbeThreads, 2048 / kProbeThreads)
     k_probe(const K* __restrict__ q, uint64_t nq, const uint32_t* __restrict__ off, const K* __restrict__ ck,
             uint32_t* __restrict__ out, uint32_t nwhole, const uint32_t* __restrict__ qpos, Map map,
-            uint64_t map_buckets) {
+            uint64_t map_buckets, uint32_t run) {
   using Reader = ReaderOf<Map>;
   map.init();
   const uint32_t last = (uintptr_t)ck % Reader::kAlign == 0 ? __ldg(off + map_buckets) : 0u;
   const uint64_t bd = blockDim.x;
   const uint64_t span = (uint64_t)gridDim.x * bd;
-  uint64_t base = (uint64_t)blockIdx.x * bd;
+  uint64_t base = (uint64_t)blockIdx.x * bd * (Map::kNeedsPos ? run : 1);
+  uint32_t left = run;
   K next = base + threadIdx.x < nq ? __ldcs(q + base + threadIdx.x) : K(0);
-  for (; base < nq; base += span) {
+  for (uint64_t step; base < nq; base += step) {
     const uint64_t i = base + threadIdx.x;
     const K key = next;
-    next = i + span < nq ? __ldcs(q + i + span) : K(0);
+    step = span;
+    if (Map::kNeedsPos) {
+      step = bd;
+      if (--left == 0) {  // on to the CTA's next run
+        left = run;
+        step = (span - bd) * run + bd;
+      }
+    }
+    next = i + step < nq ? __ldcs(q + i + step) : K(0);
     if (i >= nq) continue;
     const uint32_t b = map(key, qpos ? __ldg(qpos + i) : (uint32_t)i);
     uint32_t s, e;
@@ -165,7 +176,7 @@ __global__ void __launch_bounds__(kProbeThreads, 2048 / kProbeThreads)
 
 template <typename K, typename Map>
 hg_status probe_launch(const K* q, uint64_t nq, const uint32_t* off, const K* ck, uint32_t* out,
-                       uint64_t V, cudaStream_t st, Map map, const uint32_t* qpos) {
+                       uint64_t V, cudaStream_t st, Map map, const uint32_t* qpos, uint32_t run) {
   if (nq == 0) return HG_OK;
   // buckets whose aligned words of offsets lie inside the V+1 entries (none
   // if the array is not aligned): V + 1 <= 2^32 entries make whole words up
@@ -181,18 +192,21 @@ hg_status probe_launch(const K* q, uint64_t nq, const uint32_t* off, const K* ck
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, kern, kProbeThreads, 0) != cudaSuccess || x <= 0) x = 4;
     per_sm = x;
   }
-  const uint64_t want = (nq + kProbeThreads - 1) / kProbeThreads;
+  const uint64_t blocks = (nq + kProbeThreads - 1) / kProbeThreads;
+  // (a run only where every resident CTA has one)
+  run = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(Map::kNeedsPos ? run : 1, blocks / ((uint64_t)sms * per_sm)));
+  const uint64_t want = (blocks + run - 1) / run;
   const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)sms * per_sm));
   {
     HG_TRACE("k_probe", st);
-    kern<<<grid, kProbeThreads, 0, st>>>(q, nq, off, ck, out, nwhole, qpos, map, V);
+    kern<<<grid, kProbeThreads, 0, st>>>(q, nq, off, ck, out, nwhole, qpos, map, V, run);
   }
   return last_launch_status();
 }
 
 #define HG_INST(K, M) \
   template hg_status probe_launch<K, M>(const K*, uint64_t, const uint32_t*, const K*, uint32_t*, uint64_t, \
-                                        cudaStream_t, M, const uint32_t*);
+                                        cudaStream_t, M, const uint32_t*, uint32_t);
 HG_INST(uint32_t, MurmurMap<true>)
 HG_INST(uint64_t, MurmurMap<true>)
 HG_INST(uint32_t, MurmurMap<false>)
