@@ -132,10 +132,11 @@ hg_status hg_probe_binned(const hg_config* cfg, const hg_table* table, const voi
  * (d_keys [n], d_queries [q]), the table is built into `table` (device
  * buffers of n keys, table->n must equal n) with implicit ids, the queries
  * are probed (binned when d_probe_ws is given, else direct) into d_counts
- * [q], and the counts are copied back to h_counts [q].  Everything is
+ * [q], and the counts are copied back to h_counts [q] (many queries in up to
+ * four pieces, whose copies overlap the probes of the others).  Everything is
  * asynchronous with respect to the host (host buffers should be pinned for
  * the copies to overlap other work); h_counts is valid after `stream` is
- * synchronised.  The two host -> device copies run on a copy stream the
+ * synchronised.  The copies run on two copy streams (up and down) the
  * library keeps per device, ordered after the work already queued on
  * `stream` and joined back to `stream` by events, and the kernels of a call
  * start after those of the previous call on the same device (on whatever

@@ -1,5 +1,6 @@
 // C ABI entry points of libhg.so: argument checks, workspace layout and
 // dispatch to the kernels.  See include/hg.h for the contract.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -171,8 +172,9 @@ size_t hg_probe_workspace_size(const hg_config* cfg, uint64_t table_n, uint64_t 
   return p.total;
 }
 
-hg_status hg_probe_binned(const hg_config* cfg, const hg_table* table, const void* d_queries, uint64_t q,
-                          uint32_t* d_counts, void* d_ws, size_t ws_bytes, void* stream) {
+// hg_probe_binned; clear: the workspace's status is set back first.
+static hg_status probe_binned_call(const hg_config* cfg, const hg_table* table, const void* d_queries, uint64_t q,
+                                   uint32_t* d_counts, void* d_ws, size_t ws_bytes, void* stream, bool clear) {
   hg_status rc = validate_config(cfg);
   if (rc != HG_OK) return rc;
   if (!table || !table->d_offsets || !d_ws) return HG_ERR_INVALID_ARG;
@@ -188,7 +190,7 @@ hg_status hg_probe_binned(const hg_config* cfg, const hg_table* table, const voi
   if (!slabs && !make_probe_plan(cfg, table->n, q, &p)) return HG_ERR_UNSUPPORTED;
   if (ws_bytes < (slabs ? sp.total : p.total)) return HG_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
-  if (cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st) != cudaSuccess) return HG_ERR_CUDA;
+  if (clear && cudaMemsetAsync(d_ws, 0, sizeof(WsHeader), st) != cudaSuccess) return HG_ERR_CUDA;
   if (q == 0) return HG_OK;
   return dispatch_key_map(cfg, [&](auto k, auto map) -> hg_status {
     using K = decltype(k);
@@ -199,12 +201,17 @@ hg_status hg_probe_binned(const hg_config* cfg, const hg_table* table, const voi
   });
 }
 
+hg_status hg_probe_binned(const hg_config* cfg, const hg_table* table, const void* d_queries, uint64_t q,
+                          uint32_t* d_counts, void* d_ws, size_t ws_bytes, void* stream) {
+  return probe_binned_call(cfg, table, d_queries, q, d_counts, d_ws, ws_bytes, stream, true);
+}
+
 // Per-device state of hg_build_probe_host (created on first use, kept until
-// exit): the upload stream, on which the host -> device copies of all calls
+// exit): the upload and download streams, on which the copies of all calls
 // queue in call order, and an event marking the end of the last call's
 // kernels, after which the next call's kernels start.
 struct HostPipe {
-  cudaStream_t up = nullptr;
+  cudaStream_t up = nullptr, down = nullptr;
   cudaEvent_t done = nullptr;
   bool recorded = false;
 };
@@ -215,8 +222,9 @@ static HostPipe* host_pipe() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   HostPipe& p = pipes[dev];
   if (!p.up && cudaStreamCreateWithFlags(&p.up, cudaStreamNonBlocking) != cudaSuccess) p.up = nullptr;
+  if (!p.down && cudaStreamCreateWithFlags(&p.down, cudaStreamNonBlocking) != cudaSuccess) p.down = nullptr;
   if (!p.done && cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming) != cudaSuccess) p.done = nullptr;
-  return p.up && p.done ? &p : nullptr;
+  return p.up && p.down && p.done ? &p : nullptr;
 }
 
 // Records an event on `from` and makes `to` wait for it.
@@ -226,6 +234,30 @@ static bool join(cudaStream_t from, cudaStream_t to) {
   const bool ok = cudaEventRecord(e, from) == cudaSuccess && cudaStreamWaitEvent(to, e, 0) == cudaSuccess;
   cudaEventDestroy(e);  // released once it has completed
   return ok;
+}
+
+// Queries of one piece of a host call.  The counts of a piece go back while
+// the next piece is probed and its queries may still be on their way, so only
+// one piece's probe and download are exposed: bound by the link (1.27 ms up
+// and 0.69 ms down for 2^25 keys and queries).  Whole / 2 / 4 / 8 pieces, ms:
+// 2^25 keys and queries 2.56 / 2.27 / 2.21 / 2.45, 2^28 19.6 / 16.7 / 15.7 /
+// 15.4, 2^16 keys and 2^26 queries 3.60 / 2.60 / 2.15 / 1.96.  Pieces of 2^21
+// cost more than they hide (2^24 1.27 -> 1.46), and so do pieces much smaller
+// than the table, whose slices every piece reads again (2^28 keys, 2^25
+// queries: 10.4 whole, 10.8 in pieces of 2^23), hence n / 4.
+constexpr uint64_t kHostPieces = 4;
+constexpr uint64_t kHostPieceMin = 1ull << 22;
+static uint64_t host_piece(const hg_config* cfg, uint64_t n, uint64_t q, bool binned, size_t ws_bytes) {
+  const uint64_t piece = align_up((size_t)std::max<uint64_t>({kHostPieceMin, n / 4, (q + kHostPieces - 1) / kHostPieces}), 4096);
+  if (piece >= q || !binned) return std::min(piece, q);
+  SlabProbePlan sp{};
+  if (make_slab_probe_plan(cfg, n, q, &sp)) return q;  // (reads slab sizes back for every piece)
+  const uint64_t last = q - (q - 1) / piece * piece;
+  for (uint64_t x : {piece, last}) {
+    const size_t need = hg_probe_workspace_size(cfg, n, x);
+    if (need == 0 || need > ws_bytes) return q;
+  }
+  return piece;
 }
 
 hg_status hg_build_probe_host(const hg_config* cfg, const void* h_keys, uint64_t n, const void* h_queries,
@@ -274,21 +306,47 @@ hg_status hg_build_probe_host(const hg_config* cfg, const void* h_keys, uint64_t
   if (n > 0 && cudaMemcpyAsync(d_keys, h_keys, n * kb, cudaMemcpyHostToDevice, up) != cudaSuccess) return HG_ERR_CUDA;
   if (!join(up, st)) return HG_ERR_CUDA;
   if (pp->recorded && cudaStreamWaitEvent(st, pp->done, 0) != cudaSuccess) return HG_ERR_CUDA;
-  if (q > 0 && cudaMemcpyAsync(d_queries, h_queries, q * kb, cudaMemcpyHostToDevice, up) != cudaSuccess)
-    return HG_ERR_CUDA;
+  const uint64_t piece = q > 0 ? host_piece(cfg, n, q, d_probe_ws != nullptr, probe_ws_bytes) : 1;
+  struct Events {  // the pieces' queries have arrived
+    cudaEvent_t e[kHostPieces] = {};
+    ~Events() {
+      for (cudaEvent_t x : e)
+        if (x) cudaEventDestroy(x);  // released once it has completed
+    }
+  } here;
+  for (uint64_t x = 0, i = 0; x < q; x += piece, ++i) {
+    if (cudaMemcpyAsync((uint8_t*)d_queries + x * kb, (const uint8_t*)h_queries + x * kb,
+                        std::min(piece, q - x) * kb, cudaMemcpyHostToDevice, up) != cudaSuccess ||
+        cudaEventCreateWithFlags(&here.e[i], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventRecord(here.e[i], up) != cudaSuccess)
+      return HG_ERR_CUDA;
+  }
   // the table's buffers are this call's output (hg_table carries them as const for probes)
   rc = hg_build(cfg, d_keys, nullptr, n, const_cast<uint32_t*>(table->d_offsets), const_cast<void*>(table->d_keys),
                 const_cast<uint32_t*>(table->d_ids), d_build_ws, build_ws_bytes, stream);
   if (rc != HG_OK) return rc;
-  if (!join(up, st)) return HG_ERR_CUDA;
   if (q == 0) return HG_OK;
-  rc = d_probe_ws ? hg_probe_binned(cfg, table, d_queries, q, d_counts, d_probe_ws, probe_ws_bytes, stream)
-                  : hg_probe(cfg, table, d_queries, q, d_counts, stream);
-  if (rc != HG_OK) return rc;
-  if (cudaEventRecord(pp->done, st) != cudaSuccess) return HG_ERR_CUDA;
-  pp->recorded = true;
-  if (cudaMemcpyAsync(h_counts, d_counts, q * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) return HG_ERR_CUDA;
-  return HG_OK;
+  for (uint64_t x = 0, i = 0; x < q && rc == HG_OK; x += piece, ++i) {
+    const uint64_t m = std::min(piece, q - x);
+    const uint8_t* const dq = (const uint8_t*)d_queries + x * kb;
+    if (cudaStreamWaitEvent(st, here.e[i], 0) != cudaSuccess) {
+      rc = HG_ERR_CUDA;
+      break;
+    }
+    rc = d_probe_ws ? probe_binned_call(cfg, table, dq, m, d_counts + x, d_probe_ws, probe_ws_bytes, stream, x == 0)
+                    : hg_probe(cfg, table, dq, m, d_counts + x, stream);
+    if (rc != HG_OK) break;
+    if (x + m == q) {
+      if (cudaEventRecord(pp->done, st) == cudaSuccess) pp->recorded = true;
+      else rc = HG_ERR_CUDA;
+    }
+    if (!join(st, pp->down) ||
+        cudaMemcpyAsync(h_counts + x, d_counts + x, m * 4, cudaMemcpyDeviceToHost, pp->down) != cudaSuccess)
+      rc = HG_ERR_CUDA;
+  }
+  // the caller's stream ends after the downloads, also when the call failed on the way
+  if (!join(pp->down, st)) return HG_ERR_CUDA;
+  return rc;
 }
 
 size_t hg_join_workspace_size(const hg_config* cfg, uint64_t nA, uint64_t nB) {
