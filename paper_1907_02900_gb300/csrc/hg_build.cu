@@ -846,15 +846,17 @@ __global__ void __launch_bounds__(512) k_hist_late(PartArgs<K> a, uint32_t* __re
       if (end <= t0) continue;  // (block-uniform) an empty super-bin
       if (threadIdx.x < 256) hist[threadIdx.x] = 0;
       __syncthreads();
-      uint32_t j = t0 + threadIdx.x;
-      for (; j < end && end - j > 7 * 512; j += 8 * 512) {  // eight loads in flight
+      const K* const in = a.in_k + t0;
+      const uint32_t len = end - t0;
+      uint32_t j = threadIdx.x;
+      for (; j + 7 * 512 < len; j += 8 * 512) {  // eight loads in flight
         K k[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) k[u] = __ldcs(a.in_k + j + u * 512);
+        for (int u = 0; u < 8; ++u) k[u] = __ldcs(in + j + u * 512);
 #pragma unroll
         for (int u = 0; u < 8; ++u) atomicAdd(&hist[(map(k[u]) >> a.s) & dmask], 1u);
       }
-      for (; j < end; j += 512) atomicAdd(&hist[(map(__ldcs(a.in_k + j)) >> a.s) & dmask], 1u);
+      for (; j < len; j += 512) atomicAdd(&hist[(map(__ldcs(in + j)) >> a.s) & dmask], 1u);
       __syncthreads();
       if (threadIdx.x <= dmask && hist[threadIdx.x] != 0) atomicAdd(T + ((uint64_t)x << a.sshift) + threadIdx.x, hist[threadIdx.x]);
       __syncthreads();

@@ -64,16 +64,16 @@ struct TableReader<true> {
                                                      K key) {
     constexpr uint32_t P = 32 / sizeof(K);
     uint32_t cnt = 0;
-    for (uint32_t j = s & ~(P - 1); j < e; j += P) {
+    for (uint32_t j = s & ~(P - 1);; j += P) {
       if (last >= P && j <= last - P) {
         const Sector x = load_sector(ck + j);
 #pragma unroll
         for (uint32_t l = 0; l < P; ++l) cnt += word_key(x.w, l, K(0)) == key;
       } else {
-        for (uint32_t l = max(j, s); l < min(j + P, e); ++l) cnt += __ldg(ck + l) == key;
+        for (uint32_t l = max(j, s); l < j + min(P, e - j); ++l) cnt += __ldg(ck + l) == key;
       }
+      if (e - j <= P) return cnt;  // (j + P may be 2^32)
     }
-    return cnt;
   }
 };
 
@@ -98,22 +98,22 @@ struct TableReader<false> {
     uint32_t cnt = 0;
     if (sizeof(K) == 4 && last != 0) {
       constexpr uint32_t P = 4;
-      for (uint32_t j = s & ~(P - 1); j < e; j += P) {
+      for (uint32_t j = s & ~(P - 1);; j += P) {
         if (last >= P && j <= last - P) {
           const uint4 x = __ldg(reinterpret_cast<const uint4*>(ck + j));
           const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
           for (uint32_t l = 0; l < P; ++l) cnt += (j + l >= s) & (j + l < e) & (w[l] == key);
         } else {
-          for (uint32_t l = max(j, s); l < e; ++l) cnt += __ldg(ck + l) == key;
+          for (uint32_t l = max(j, s); l < j + min(P, e - j); ++l) cnt += __ldg(ck + l) == key;
         }
+        if (e - j <= P) return cnt;
       }
-      return cnt;
     }
     cnt = __ldg(ck + s) == key;
     uint32_t j = s + 1;
     // four independent loads in flight per round for long buckets
-    for (; j + 4 <= e; j += 4) {
+    for (; e - j >= 4; j += 4) {
       const K a0 = __ldg(ck + j), a1 = __ldg(ck + j + 1), a2 = __ldg(ck + j + 2), a3 = __ldg(ck + j + 3);
       cnt += (a0 == key) + (a1 == key) + (a2 == key) + (a3 == key);
     }
