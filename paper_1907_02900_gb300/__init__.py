@@ -311,8 +311,8 @@ def probe(table: Table, queries, stream=None, binned: bool | None = None, ws=Non
     counts = torch.empty(q, dtype=torch.uint32, device=queries.device)
     if binned is None:
         binned = _binning_pays(table, q)
-        if not binned and q >= 1 << 20 and queries.data_ptr() % 16:
-            raise HGError(1, "hg_probe")  # large batches are 16-byte aligned, whichever probe takes them
+        if not binned and q >= 1 << 20 and (queries.data_ptr() % 16 or q >= 1 << 32):
+            raise HGError(1, "hg_probe")  # large batches: 16-byte aligned, below 2^32, whichever probe takes them
     if binned:
         need = probe_workspace_size(table, q)
         if need == 0:
